@@ -1,11 +1,13 @@
 // ray.cu - parallel-beam ray transform (the forward operator of the
 // learned primal-dual reconstruction of Sec. 4.4) and its exact transpose.
 //
-//   k_ray_forward  one thread per ray (image, angle, bin): Joseph's method,
-//                  one linear-interpolation sample per pixel row (or column).
-//   k_ray_adjoint  one thread per pixel: for each angle, the 2-3 bins whose
-//                  rays sample this pixel's row (column) near it, with the
-//                  forward's own weights.
+//   k_ray_forward  a CTA takes 256 bins of up to two neighbouring angles and up
+//                  to four images: Joseph's method, one linear-interpolation
+//                  sample per pixel row (or column), the rows it samples
+//                  staged in shared memory with the images interleaved.
+//   k_ray_adjoint  two pixels and up to four images per thread: for each angle,
+//                  the bins whose rays sample this pixel's row (column) near
+//                  it, with the forward's own weights.
 //
 // Sampling of angle a: the ray of bin d meets row (column) t of the image at
 // the fractional pixel coordinate u = A_a d + B_a t + C_a along that row
@@ -30,71 +32,216 @@ namespace {
 struct AngleParam {
   float A, B, C, w;   // u = A d + B t + C; sample weight w
   int by_rows;        // 1: sample t is a pixel row (|cos phi| >= |sin phi|)
-  int pad[3];
+  float inv_a;        // 1 / A
+  int bins;           // adjoint: bins from floor(d - 1/|A| - ADJ_MARGIN) on that hold
+                      // every bin with |u - k| < 1 around the fractional bin d
+  int pad;
 };
+static_assert(sizeof(AngleParam) == 32, "read as two float4");
 
-__device__ __forceinline__ float sample_u(const AngleParam& q, int d, int t) {
-  return fmaf(q.A, (float)d, fmaf(q.B, (float)t, q.C));
+__device__ __forceinline__ AngleParam load_angle(const AngleParam* p) {
+  const float4 lo = __ldg(reinterpret_cast<const float4*>(p));
+  const float4 hi = __ldg(reinterpret_cast<const float4*>(p) + 1);
+  AngleParam q;
+  q.A = lo.x; q.B = lo.y; q.C = lo.z; q.w = lo.w;
+  q.by_rows = __float_as_int(hi.x); q.inv_a = hi.y; q.bins = __float_as_int(hi.z); q.pad = 0;
+  return q;
 }
 
-__global__ void __launch_bounds__(256) k_ray_forward(const float* __restrict__ img,
-                                                     float* __restrict__ sino,
-                                                     const AngleParam* __restrict__ prm, int n,
-                                                     int A, int D) {
-  const int d = blockIdx.x * blockDim.x + threadIdx.x;
-  const int a = blockIdx.y;
-  if (d >= D) return;
-  const AngleParam q = prm[a];
-  const float* f = img + (size_t)blockIdx.z * n * n;
-  float acc = 0.f;
-  for (int t = 0; t < n; ++t) {
-    const float u = sample_u(q, d, t);
-    const float fk = floorf(u);
-    if (fk < -1.f || fk > (float)(n - 1)) continue;   // both neighbours outside
-    const int k0 = (int)fk;
-    const float w1 = u - fk, w0 = 1.f - w1;
-    float v0 = 0.f, v1 = 0.f;
-    if (q.by_rows) {
-      if (k0 >= 0) v0 = __ldg(f + (size_t)t * n + k0);
-      if (k0 + 1 < n) v1 = __ldg(f + (size_t)t * n + k0 + 1);
-    } else {
-      if (k0 >= 0) v0 = __ldg(f + (size_t)k0 * n + t);
-      if (k0 + 1 < n) v1 = __ldg(f + (size_t)(k0 + 1) * n + t);
+__device__ __forceinline__ float sample_u(const AngleParam& q, float d, float t) {
+  return fmaf(q.A, d, fmaf(q.B, t, q.C));
+}
+
+// Integer nearest to x (ties to even) for |x| < 2^22, as float and int, by
+// adding and subtracting 1.5 * 2^23 (two float additions; floorf and the
+// conversion run at a quarter of their rate).  With x = u - 1/2 it is floor(u),
+// or u - 1 for some integer u, where the weights 0 and 1 then name the same
+// pixel.
+__device__ __forceinline__ float round_near(float x, int* i) {
+  const float m = x + 12582912.f;
+  *i = __float_as_int(m) - 0x4B400000;
+  return m - 12582912.f;
+}
+
+template <int NB> struct Vec;
+template <> struct Vec<1> { float v[1]; };
+template <> struct __align__(8) Vec<2> { float v[2]; };
+template <> struct __align__(16) Vec<4> { float v[4]; };
+
+// ---------------------------------------------------------------- forward
+// What bounds it: shared-memory reads, two NB-wide words per sample.  Reading
+// the image through L1 instead, one ray per thread, cost a gather of up to 32
+// lines per load at the angles sampled by columns; staging T rows (or, transposed,
+// T columns) of the pixels that the CTA's rays cross makes both kinds of angle
+// the same, interleaving NB images shares the position and the weights between
+// them, and two neighbouring angles share one staging.  Measured at 8 images of
+// 512 x 512, 180 angles, 725 bins: 1402 us with one thread per ray, 338 us so (one
+// image: 239 and 187 us).
+constexpr int FWD_BINS = 256;      // bins (threads) per CTA
+constexpr int FWD_ANGLES = 2;      // most angles per CTA
+constexpr int FWD_ROWS = 8;        // most samples t staged at a time
+constexpr size_t FWD_SMEM = 56 * 1024;   // four CTAs per SM
+
+struct AngleGroup { int a0, na; };   // neighbouring angles of one kind
+
+template <int NB>
+__global__ void __launch_bounds__(FWD_BINS) k_ray_forward(const float* __restrict__ img,
+                                                          float* __restrict__ sino,
+                                                          const AngleParam* __restrict__ prm,
+                                                          const AngleGroup* __restrict__ groups,
+                                                          int n, int A, int D, int B, int T, int pitch) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  Vec<NB>* S = reinterpret_cast<Vec<NB>*>(smem);     // [T][pitch]
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const AngleGroup grp = groups[blockIdx.y];
+  const int d_lo = blockIdx.x * FWD_BINS, d_hi = min(D - 1, d_lo + FWD_BINS - 1);
+  const int d = d_lo + tid, b0 = blockIdx.z * NB;
+  const float df = (float)min(d, d_hi);
+  AngleParam q[FWD_ANGLES];
+#pragma unroll
+  for (int k = 0; k < FWD_ANGLES; ++k) q[k] = load_angle(prm + grp.a0 + min(k, grp.na - 1));
+  const bool by_rows = q[0].by_rows != 0;
+  const float* f[NB];
+#pragma unroll
+  for (int b = 0; b < NB; ++b) f[b] = img + (size_t)min(b0 + b, B - 1) * n * n;
+  float acc[FWD_ANGLES][NB];
+#pragma unroll
+  for (int k = 0; k < FWD_ANGLES; ++k)
+#pragma unroll
+    for (int b = 0; b < NB; ++b) acc[k][b] = 0.f;
+
+  for (int t0 = 0; t0 < n; t0 += T) {
+    const int tn = min(T, n - t0);
+    // pixels that the block's samples can touch: u is monotone in d and in t
+    float lo = 1e30f, hi = -1e30f;
+#pragma unroll
+    for (int k = 0; k < FWD_ANGLES; ++k) {
+      const float da = (float)(q[k].A >= 0.f ? d_lo : d_hi), db = (float)(q[k].A >= 0.f ? d_hi : d_lo);
+      const float ta = (float)(q[k].B >= 0.f ? t0 : t0 + tn - 1), tb = (float)(q[k].B >= 0.f ? t0 + tn - 1 : t0);
+      lo = fminf(lo, sample_u(q[k], da, ta));
+      hi = fmaxf(hi, sample_u(q[k], db, tb));
     }
-    acc = fmaf(w0, v0, fmaf(w1, v1, acc));
+    if (hi < -1.f || lo > (float)n) continue;        // every sample outside (the whole CTA agrees)
+    // two zero pixels on either side stand for everything outside the image
+    const int k_lo = max(-2, (int)floorf(fmaxf(lo, -4.f)) - 1);
+    const int k_hi = min(n + 1, (int)floorf(fminf(hi, (float)(n + 4))) + 1);
+    const int width = min(k_hi - k_lo + 1, pitch);
+    __syncthreads();                                 // the earlier rows have been read
+    if (by_rows) {
+      for (int tt = warp; tt < tn; tt += FWD_BINS / 32)
+        for (int x = lane; x < width; x += 32) {
+          const int k = k_lo + x;
+          Vec<NB> v;
+#pragma unroll
+          for (int b = 0; b < NB; ++b)
+            v.v[b] = k >= 0 && k < n ? __ldg(f[b] + (size_t)(t0 + tt) * n + k) : 0.f;
+          S[tt * pitch + x] = v;
+        }
+    } else {
+      const int tt = lane & (FWD_ROWS - 1);          // FWD_ROWS consecutive columns of a pixel row
+      for (int x = warp * (32 / FWD_ROWS) + lane / FWD_ROWS; x < width; x += FWD_BINS / FWD_ROWS) {
+        const int k = k_lo + x;
+        Vec<NB> v;
+#pragma unroll
+        for (int b = 0; b < NB; ++b)
+          v.v[b] = k >= 0 && k < n && tt < tn ? __ldg(f[b] + (size_t)k * n + t0 + tt) : 0.f;
+        if (tt < tn) S[tt * pitch + x] = v;
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < FWD_ANGLES; ++k) {
+      if (k >= grp.na) break;
+      const float ua = sample_u(q[k], df, (float)t0), ub = sample_u(q[k], df, (float)(t0 + tn - 1));
+      if (!__any_sync(0xffffffffu, fmaxf(ua, ub) >= -1.f && fminf(ua, ub) <= (float)n)) continue;
+#pragma unroll 4
+      for (int tt = 0; tt < tn; ++tt) {
+        const float u = sample_u(q[k], df, (float)(t0 + tt));
+        int i;
+        const float w1 = u - round_near(u - 0.5f, &i), w0 = 1.f - w1;
+        const Vec<NB>* s = S + tt * pitch + min(max(i - k_lo, 0), width - 2);
+        const Vec<NB> v0 = s[0], v1 = s[1];
+#pragma unroll
+        for (int b = 0; b < NB; ++b) acc[k][b] = fmaf(w0, v0.v[b], fmaf(w1, v1.v[b], acc[k][b]));
+      }
+    }
   }
-  sino[((size_t)blockIdx.z * A + a) * D + d] = acc * q.w;
+  if (d > d_hi) return;
+#pragma unroll
+  for (int k = 0; k < FWD_ANGLES; ++k)
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+      if (k < grp.na && b0 + b < B)
+        sino[((size_t)(b0 + b) * A + grp.a0 + k) * D + d] = acc[k][b] * q[k].w;
 }
 
+// ---------------------------------------------------------------- adjoint
+// Pixel (t, k) of angle a receives every bin d with |u(d, t) - k| < 1, with the
+// hat weight 1 - |u - k|: exactly the forward's 1 - w1 or w1, since u - k and
+// the difference from 1 on the far side are exact in float32.  The bins start at
+// the one below the fractional bin of u = k - 1; ADJ_MARGIN covers the rounding
+// of that bin (below 0.01 over the accepted sizes).  What bounds it: issue, about
+// 50 instructions per pixel and angle for four images, whose position, weights
+// and address they share.  Measured as above: 1770 us with one thread
+// per pixel and image (a floor and a compare per candidate bin), 527 us so; 32
+// images of 128 x 128 at 30 angles: 96 and 33 us (forward 107 and 45 us).
+constexpr float ADJ_MARGIN = 0.05f;
+constexpr int ADJ_PIX = 2;         // pixels per thread, 8 rows apart
+
+template <int NB>
 __global__ void __launch_bounds__(256) k_ray_adjoint(const float* __restrict__ sino,
                                                      float* __restrict__ img,
                                                      const AngleParam* __restrict__ prm, int n,
-                                                     int A, int D) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  const int i = blockIdx.y;
-  if (j >= n) return;
-  const float* p = sino + (size_t)blockIdx.z * A * D;
-  float acc = 0.f;
+                                                     int A, int D, int B) {
+  const int j = blockIdx.x * 32 + (threadIdx.x & 31);
+  const int i0 = blockIdx.y * (8 * ADJ_PIX) + (threadIdx.x >> 5), b0 = blockIdx.z * NB;
+  const float* p[NB];
+#pragma unroll
+  for (int b = 0; b < NB; ++b) p[b] = sino + (size_t)min(b0 + b, B - 1) * A * D;
+  float acc[ADJ_PIX][NB];
+#pragma unroll
+  for (int x = 0; x < ADJ_PIX; ++x)
+#pragma unroll
+    for (int b = 0; b < NB; ++b) acc[x][b] = 0.f;
   for (int a = 0; a < A; ++a) {
-    const AngleParam q = prm[a];
-    const int t = q.by_rows ? i : j, k = q.by_rows ? j : i;
-    // bins whose u at sample t lies in (k - 1, k + 1): d near (k - B t - C) / A
-    const float dc = ((float)k - fmaf(q.B, (float)t, q.C)) / q.A;
-    const float half = 1.f / fabsf(q.A);
-    const int lo = max(0, (int)floorf(dc - half) - 1);
-    const int hi = min(D - 1, (int)ceilf(dc + half) + 1);
-    float sa = 0.f;
-    for (int d = lo; d <= hi; ++d) {
-      const float u = sample_u(q, d, t);
-      const float fk = floorf(u);
-      const float w1 = u - fk;
-      const int k0 = (int)fk;
-      if (k0 == k) sa = fmaf(1.f - w1, __ldg(p + (size_t)a * D + d), sa);
-      else if (k0 + 1 == k) sa = fmaf(w1, __ldg(p + (size_t)a * D + d), sa);
+    const AngleParam q = load_angle(prm + a);
+    const float first = fabsf(q.inv_a) + (ADJ_MARGIN + 0.5f);
+    const int row = a * D;
+#pragma unroll
+    for (int x = 0; x < ADJ_PIX; ++x) {
+      const int i = i0 + 8 * x;
+      const float t = (float)(q.by_rows ? i : j), k = (float)(q.by_rows ? j : i);
+      const float base = fmaf(q.B, t, q.C);
+      int lo;
+      const float flo = round_near(fminf(fmaxf((k - base) * q.inv_a - first, -1e6f), 1e6f), &lo);
+      float sa[NB];
+#pragma unroll
+      for (int b = 0; b < NB; ++b) sa[b] = 0.f;
+      auto bin = [&](int m) {
+        const float w = __saturatef(1.f - fabsf(fmaf(q.A, flo + (float)m, base) - k));
+        if (w > 0.f) {               // a bin outside the hat is not read into the sum
+#pragma unroll
+          for (int b = 0; b < NB; ++b) sa[b] = fmaf(w, __ldg(p[b] + (row + lo + m)), sa[b]);
+        }
+      };
+      if (lo >= 0 && lo + q.bins <= D) {
+        bin(0);
+        bin(1);
+        if (q.bins > 2) bin(2);
+        for (int m = 3; m < q.bins; ++m) bin(m);
+      } else {
+        for (int m = max(0, -lo); m < q.bins && lo + m < D; ++m) bin(m);
+      }
+#pragma unroll
+      for (int b = 0; b < NB; ++b) acc[x][b] = fmaf(sa[b], q.w, acc[x][b]);
     }
-    acc = fmaf(sa, q.w, acc);
   }
-  img[((size_t)blockIdx.z * n + i) * n + j] = acc;
+#pragma unroll
+  for (int x = 0; x < ADJ_PIX; ++x)
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+      if (j < n && i0 + 8 * x < n && b0 + b < B)
+        img[((size_t)(b0 + b) * n + i0 + 8 * x) * n + j] = acc[x][b];
 }
 
 bool aligned4(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 3u) == 0; }
@@ -104,7 +251,56 @@ bool aligned4(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 3u) == 0
 struct shl_ray {
   int device = 0, n = 0, A = 0, D = 0;
   AngleParam* dPrm = nullptr;
+  AngleGroup* dGrp = nullptr;
+  int ngrp = 0;
+  double a_max = 0, b_max = 0;      // largest |A| and |B| over the angles
+  double pair_max = 0;              // largest |u - u'| between the angles of a group
 };
+
+namespace {
+
+// Images per CTA: the position and the weights of a sample are shared by the
+// images, so as many as there are (up to four) unless the launch would then
+// leave SMs without two CTAs.
+int images_per_cta(long long ctas_per_image, int batch) {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  for (int nb = 4; nb > 1; nb /= 2)
+    if (batch >= nb && ctas_per_image * ((batch + nb - 1) / nb) >= 2LL * sms) return nb;
+  return 1;
+}
+
+template <int NB>
+cudaError_t forward_nb(const shl_ray* op, const float* img, int batch, float* sino, cudaStream_t st) {
+  // staged pixels per sample row: what FWD_BINS bins and T rows can reach, at
+  // most the whole row with its zero pixels; odd, so that the transposed stores
+  // of the column-sampled angles meet no bank twice
+  int T = FWD_ROWS, pitch = 0;
+  for (;; T /= 2) {
+    const double reach = (FWD_BINS - 1.0) * op->a_max + (T - 1.0) * op->b_max + op->pair_max + 8.0;
+    pitch = (reach < op->n + 4.0 ? (int)reach : op->n + 4) | 1;
+    if ((size_t)T * pitch * sizeof(Vec<NB>) <= FWD_SMEM || T == 1) break;
+  }
+  const size_t smem = (size_t)T * pitch * sizeof(Vec<NB>);
+  cudaError_t e = cudaSuccess;
+  if (smem > 48 * 1024)
+    e = cudaFuncSetAttribute(k_ray_forward<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e) return e;
+  const dim3 grid((op->D + FWD_BINS - 1) / FWD_BINS, op->ngrp, (batch + NB - 1) / NB);
+  k_ray_forward<NB><<<grid, FWD_BINS, smem, st>>>(img, sino, op->dPrm, op->dGrp, op->n, op->A, op->D,
+                                                  batch, T, pitch);
+  return cudaGetLastError();
+}
+
+template <int NB>
+cudaError_t adjoint_nb(const shl_ray* op, const float* sino, int batch, float* img, cudaStream_t st) {
+  const dim3 grid((op->n + 31) / 32, (op->n + 8 * ADJ_PIX - 1) / (8 * ADJ_PIX), (batch + NB - 1) / NB);
+  k_ray_adjoint<NB><<<grid, 256, 0, st>>>(sino, img, op->dPrm, op->n, op->A, op->D, batch);
+  return cudaGetLastError();
+}
+
+}  // namespace
 
 extern "C" {
 
@@ -130,17 +326,50 @@ shl_status shl_ray_create(int n, int n_angles, int n_det, int device, shl_ray** 
     q.B = (float)(-h * other / den);
     q.C = (float)((-S + 0.5 * ds + other * (1.0 - 0.5 * h)) / den + 1.0 / h - 0.5);
     q.w = (float)(h / std::fabs(q.by_rows ? c : s));
+    q.inv_a = (float)(den / ds);
+    q.bins = (int)std::floor(2.0 * std::fabs(den / ds) + 2.0 * ADJ_MARGIN) + 2;
+  }
+  // the forward's groups: two neighbouring angles share a staging when the pixels
+  // they sample stay within PAIR_PIXELS of each other (u is affine in d and t, so
+  // the corners bound the difference)
+  constexpr double PAIR_PIXELS = 64.0;
+  std::vector<AngleGroup> grp;
+  double a_max = 0, b_max = 0, pair_max = 0;
+  for (const AngleParam& q : prm) {
+    a_max = std::max(a_max, (double)std::fabs(q.A));
+    b_max = std::max(b_max, (double)std::fabs(q.B));
+  }
+  for (int a = 0; a < n_angles;) {
+    double gap = 1e30;
+    if (a + 1 < n_angles && prm[a].by_rows == prm[a + 1].by_rows) {
+      gap = 0;
+      for (int c = 0; c < 4; ++c) {
+        const double d = c & 1 ? n_det - 1.0 : 0.0, t = c & 2 ? n - 1.0 : 0.0;
+        gap = std::max(gap, std::fabs(((double)prm[a].A - prm[a + 1].A) * d +
+                                      ((double)prm[a].B - prm[a + 1].B) * t +
+                                      ((double)prm[a].C - prm[a + 1].C)));
+      }
+    }
+    const int na = gap <= PAIR_PIXELS ? FWD_ANGLES : 1;
+    if (na > 1) pair_max = std::max(pair_max, gap);
+    grp.push_back({a, na});
+    a += na;
   }
   int prev = -1;
   cudaGetDevice(&prev);
   if (prev != device) cudaSetDevice(device);
   shl_ray* op = new shl_ray;
   op->device = device; op->n = n; op->A = n_angles; op->D = n_det;
+  op->ngrp = (int)grp.size();
+  op->a_max = a_max; op->b_max = b_max; op->pair_max = pair_max;
   cudaError_t e = cudaMalloc(&op->dPrm, sizeof(AngleParam) * n_angles);
+  if (!e) e = cudaMalloc(&op->dGrp, sizeof(AngleGroup) * grp.size());
   if (!e) e = cudaMemcpy(op->dPrm, prm.data(), sizeof(AngleParam) * n_angles, cudaMemcpyHostToDevice);
+  if (!e) e = cudaMemcpy(op->dGrp, grp.data(), sizeof(AngleGroup) * grp.size(), cudaMemcpyHostToDevice);
   if (prev >= 0 && prev != device) cudaSetDevice(prev);
   if (e) {
     if (op->dPrm) cudaFree(op->dPrm);
+    if (op->dGrp) cudaFree(op->dGrp);
     delete op;
     cudaGetLastError();
     return shl::set_error(e == cudaErrorMemoryAllocation ? SHL_ENOMEM : SHL_ECUDA,
@@ -156,6 +385,7 @@ shl_status shl_ray_destroy(shl_ray* op) {
   cudaGetDevice(&prev);
   if (prev != op->device) cudaSetDevice(op->device);
   cudaFree(op->dPrm);
+  cudaFree(op->dGrp);
   if (prev >= 0 && prev != op->device) cudaSetDevice(prev);
   delete op;
   return SHL_OK;
@@ -182,11 +412,14 @@ shl_status shl_ray_forward(const shl_ray* op, const float* img, int batch, float
   cudaError_t e = cudaSuccess;
   for (int b0 = 0; b0 < batch && !e; b0 += 65535) {
     const int nb = std::min(65535, batch - b0);
-    k_ray_forward<<<dim3((op->D + 255) / 256, op->A, nb), 256, 0,
-                    static_cast<cudaStream_t>(stream)>>>(img + (size_t)b0 * op->n * op->n,
-                                                         sino + (size_t)b0 * op->A * op->D,
-                                                         op->dPrm, op->n, op->A, op->D);
-    e = cudaGetLastError();
+    const float* x = img + (size_t)b0 * op->n * op->n;
+    float* y = sino + (size_t)b0 * op->A * op->D;
+    const cudaStream_t st = static_cast<cudaStream_t>(stream);
+    switch (images_per_cta((op->D + FWD_BINS - 1LL) / FWD_BINS * op->ngrp, nb)) {
+      case 4: e = forward_nb<4>(op, x, nb, y, st); break;
+      case 2: e = forward_nb<2>(op, x, nb, y, st); break;
+      default: e = forward_nb<1>(op, x, nb, y, st); break;
+    }
   }
   if (prev >= 0 && prev != op->device) cudaSetDevice(prev);
   return e ? shl::set_error(SHL_ECUDA, cudaGetErrorString(e)) : SHL_OK;
@@ -205,11 +438,14 @@ shl_status shl_ray_adjoint(const shl_ray* op, const float* sino, int batch, floa
   cudaError_t e = cudaSuccess;
   for (int b0 = 0; b0 < batch && !e; b0 += 65535) {
     const int nb = std::min(65535, batch - b0);
-    k_ray_adjoint<<<dim3((op->n + 255) / 256, op->n, nb), 256, 0,
-                    static_cast<cudaStream_t>(stream)>>>(sino + (size_t)b0 * op->A * op->D,
-                                                         img + (size_t)b0 * op->n * op->n,
-                                                         op->dPrm, op->n, op->A, op->D);
-    e = cudaGetLastError();
+    const float* y = sino + (size_t)b0 * op->A * op->D;
+    float* x = img + (size_t)b0 * op->n * op->n;
+    const cudaStream_t st = static_cast<cudaStream_t>(stream);
+    switch (images_per_cta((op->n + 31LL) / 32 * ((op->n + 8 * ADJ_PIX - 1) / (8 * ADJ_PIX)), nb)) {
+      case 4: e = adjoint_nb<4>(op, y, nb, x, st); break;
+      case 2: e = adjoint_nb<2>(op, y, nb, x, st); break;
+      default: e = adjoint_nb<1>(op, y, nb, x, st); break;
+    }
   }
   if (prev >= 0 && prev != op->device) cudaSetDevice(prev);
   return e ? shl::set_error(SHL_ECUDA, cudaGetErrorString(e)) : SHL_OK;
