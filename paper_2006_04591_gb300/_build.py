@@ -24,7 +24,7 @@ NVCC = os.path.join(CUDA_HOME, "bin", "nvcc")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 CU_SOURCES = ["fast.cu", "fused.cu", "general.cu", "noalloc.cu", "nn.cu", "nn_tc.cu", "bank_gpu.cu", "ray.cu",
-              "tc_dft.cu"]
+              "tc_dft.cu"] + ["general_pairs.cu:%d" % k for k in range(8)]   # name:part
 CPP_SOURCES = ["api.cpp", "bank_build.cpp"]
 # The checked library: every source again with -DSHL_CHECKED (bounds guards
 # with a device error word in the transform kernels), the same C ABI.
@@ -54,9 +54,11 @@ def _jobs(cu, cpp, tag, defines, verbose):
     inc = ["-I" + os.path.join(ROOT, "include"), "-I" + CSRC]
     jobs = []
     for s in cu:
-        o = os.path.join(BUILD, tag + s + ".o")
+        o = os.path.join(BUILD, tag + s.replace(":", "_") + ".o")
+        src, _, part = s.partition(":")
         jobs.append((o, [NVCC, *ARCH, "-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC",
-                         "--expt-relaxed-constexpr", *defines, *inc, "-c", os.path.join(CSRC, s),
+                         "--expt-relaxed-constexpr", *defines, *inc,
+                         *(["-DSHL_PART=" + part] if part else []), "-c", os.path.join(CSRC, src),
                          "-o", o] + (["-Xptxas", "-v"] if verbose else [])))
     gxx = shutil.which("g++") or "g++"
     for s in cpp:

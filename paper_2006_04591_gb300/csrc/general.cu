@@ -1,5 +1,6 @@
 // general.cu - transform kernels for any image size and for complex
-// Hermitian filter spectra: the decomposition, reconstruction and adjoint of
+// Hermitian filter spectra (lengths A B with A, B <= 32, and Bluestein lengths up to
+// 512: general_pairs.cuh): the decomposition, reconstruction and adjoint of
 // Sec. 3.4 on row-major half-spectrum planes [N][M/2+1] in natural DFT order
 // (real images and Hermitian filters give Hermitian spectra, so columns
 // 0..M/2 determine the rest).
@@ -45,9 +46,17 @@
 #include <complex>
 
 #include "general.h"
+#include "general_pairs_list.h"
 
 namespace shl {
 namespace gen {
+
+#define SHL_PART_DECL(K, C)                                                              \
+  cudaError_t pair_rows_part##K(int kind, const PairRowArgs& a, cudaStream_t st);        \
+  cudaError_t pair_cols_part##C(int planes, const PairColArgs& a, cudaStream_t st);
+SHL_PART_DECL(0, 4) SHL_PART_DECL(1, 5) SHL_PART_DECL(2, 6) SHL_PART_DECL(3, 7)
+#undef SHL_PART_DECL
+
 namespace {
 
 constexpr int ROW_THREADS = 256;
@@ -637,6 +646,52 @@ int largest_prime_factor(int n) {
   return n > 1 ? std::max(big, n) : big;
 }
 
+// Which part of the pair list holds (A, B, bluestein); -1: none does.
+int pair_part(int A, int B, bool bl) {
+#define SHL_FIND(K) SHL_PAIRS_##K(X)
+#define X(RA, RB, BL) if (A == RA && B == RB && bl == BL) return 0;
+  SHL_FIND(0)
+#undef X
+#define X(RA, RB, BL) if (A == RA && B == RB && bl == BL) return 1;
+  SHL_FIND(1)
+#undef X
+#define X(RA, RB, BL) if (A == RA && B == RB && bl == BL) return 2;
+  SHL_FIND(2)
+#undef X
+#define X(RA, RB, BL) if (A == RA && B == RB && bl == BL) return 3;
+  SHL_FIND(3)
+#undef X
+#undef SHL_FIND
+  return -1;
+}
+
+// The pair for lines of length L: L itself where it is one of the products; else,
+// where L has a prime factor above BLUESTEIN_PRIME (the one-output-per-thread stages
+// of this file), the shortest Bluestein length.  A = 0 otherwise.  Lengths with
+// factors up to 7 only and no pair keep the direct stages: at 350 rows these take
+// 9.1 (decomposition) and 17.9 (reconstruction) ns per thousand elements, Bluestein
+// at 222 rows 11.9 and 14.3.
+constexpr int BLUESTEIN_PRIME = 7;
+PairPlan find_pair(int L) {
+  PairPlan p{};
+  p.L = L;
+#define X(RA, RB, BL) if (!BL && RA * RB == L) { p.A = RA; p.B = RB; }
+  SHL_PAIRS_ALL(X)
+#undef X
+  if (p.A || largest_prime_factor(L) <= BLUESTEIN_PRIME) return p;
+  int best = 0;
+#define X(RA, RB, BL)                                                                \
+  if (BL && RA * RB >= 2 * L - 1 && (!best || RA * RB < best)) {                     \
+    best = RA * RB;                                                                  \
+    p.A = RA;                                                                        \
+    p.B = RB;                                                                        \
+  }
+  SHL_PAIRS_ALL(X)
+#undef X
+  p.bluestein = best != 0;
+  return p;
+}
+
 // Launches k, first raising its dynamic shared-memory limit to what this
 // launch asks for (the attribute is per function and device; a launch that
 // needs no more than the default 48 KB leaves it alone).
@@ -673,39 +728,86 @@ int col_lines(const LinePlan& pn, int W) {
   return std::min(c, W);
 }
 
+// Subband groups per image of the reconstruction: about four waves of CTAs with
+// at least ceil(K / 16) subbands a group, so that one image's K transforms are
+// spread over the GPU instead of running in one CTA.
+int rec_groups(long long ctas, long long per_sm, int subbands) {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const long long want = 4LL * std::max(sms, 1) * per_sm;
+  const long long base = std::max<long long>(1, ctas);
+  return (int)std::max<long long>(1, std::min<long long>({(want + base - 1) / base, 16, subbands}));
+}
+
 }  // namespace
+
+// Forward DFT in float64 of any length: radix 2 where it is a power of two, else
+// through a power-of-two convolution (Bluestein).
+static void dft_any(std::vector<cd>& x) {
+  const long long n = (long long)x.size();
+  if ((n & (n - 1)) == 0) {
+    fft_pow2(x, -1);
+    return;
+  }
+  size_t m = 1;
+  while ((long long)m < 2 * n - 1) m <<= 1;
+  std::vector<cd> c(n), a(m, cd(0, 0)), h(m, cd(0, 0));
+  for (long long k = 0; k < n; ++k) {
+    const double t = -PI * (double)((k * k) % (2 * n)) / (double)n;
+    c[k] = cd(std::cos(t), std::sin(t));
+    a[k] = x[k] * c[k];
+    h[k] = std::conj(c[k]);
+    if (k) h[m - k] = std::conj(c[k]);
+  }
+  fft_pow2(a, -1);
+  fft_pow2(h, -1);
+  for (size_t k = 0; k < m; ++k) a[k] *= h[k];
+  fft_pow2(a, +1);
+  for (long long k = 0; k < n; ++k) x[k] = c[k] * a[k] / (double)m;
+}
 
 LineTables make_line_tables(int L) {
   LineTables t;
   LinePlan& p = t.plan;
   p = LinePlan{};
   p.L = L;
-  p.bluestein = largest_prime_factor(L) > MAX_DIRECT_PRIME;
-  p.P = L;
-  if (p.bluestein) {
+  p.pair = find_pair(L);
+  const PairPlan& q = p.pair;
+  p.bluestein = q.A ? q.bluestein : largest_prime_factor(L) > MAX_DIRECT_PRIME;
+  p.P = q.A ? q.A * q.B : L;
+  if (p.bluestein && !q.A) {
     p.P = 1;
     while (p.P < 2 * L - 1) p.P <<= 1;
   }
-  radices_of(p.P, &p);
   const int P = p.P;
+  auto root = [&](long long k, long long n) {
+    const double a = -2.0 * PI * (double)(k % n) / (double)n;
+    t.data.push_back(make_float2((float)std::cos(a), (float)std::sin(a)));
+  };
   t.off_tw = 0;
-  t.data.resize(P);
-  for (int q = 0; q < P; ++q) {
-    const double a = -2.0 * PI * q / P;
-    t.data[q] = make_float2((float)std::cos(a), (float)std::sin(a));
+  if (q.A) {
+    for (int m = 1; m < q.B; ++m)
+      for (int k = 0; k < q.A; ++k) root((long long)m * k, P);
+    t.off_ba = t.data.size();
+    for (int m = 1; m < q.A; ++m)
+      for (int k = 0; k < q.B; ++k) root((long long)m * k, P);
+  } else {
+    radices_of(p.P, &p);
+    for (int k = 0; k < P; ++k) root(k, P);
   }
   if (p.bluestein) {
     std::vector<cd> c(L), h(P, cd(0.0, 0.0));
     for (int n = 0; n < L; ++n) {
-      const long long q = ((long long)n * n) % (2LL * L);   // exp(-i pi n^2 / L), reduced
-      const double a = -PI * (double)q / L;
+      const long long s = ((long long)n * n) % (2LL * L);   // exp(-i pi n^2 / L), reduced
+      const double a = -PI * (double)s / L;
       c[n] = cd(std::cos(a), std::sin(a));
     }
     for (int m = 0; m < L; ++m) {
       h[m] = std::conj(c[m]);
       if (m) h[P - m] = std::conj(c[m]);
     }
-    fft_pow2(h, -1);
+    dft_any(h);
     t.off_chirp = t.data.size();
     for (int n = 0; n < L; ++n) t.data.push_back(to_f2(c[n]));
     t.off_kern = t.data.size();
@@ -714,15 +816,44 @@ LineTables make_line_tables(int L) {
   return t;
 }
 
+cudaError_t launch_pair_rows(int kind, const PairRowArgs& a, cudaStream_t st) {
+  switch (pair_part(a.p.A, a.p.B, a.p.bluestein != 0)) {
+    case 0: return pair_rows_part0(kind, a, st);
+    case 1: return pair_rows_part1(kind, a, st);
+    case 2: return pair_rows_part2(kind, a, st);
+    case 3: return pair_rows_part3(kind, a, st);
+  }
+  return cudaErrorInvalidValue;
+}
+cudaError_t launch_pair_cols(int planes, const PairColArgs& a, cudaStream_t st) {
+  switch (pair_part(a.p.A, a.p.B, a.p.bluestein != 0)) {
+    case 0: return pair_cols_part4(planes, a, st);
+    case 1: return pair_cols_part5(planes, a, st);
+    case 2: return pair_cols_part6(planes, a, st);
+    case 3: return pair_cols_part7(planes, a, st);
+  }
+  return cudaErrorInvalidValue;
+}
+
 void place_line_tables(LineTables* t, const float2* dev) {
   t->plan.tw = dev + t->off_tw;
   t->plan.chirp = t->plan.bluestein ? dev + t->off_chirp : nullptr;
   t->plan.kern = t->plan.bluestein ? dev + t->off_kern : nullptr;
+  t->plan.pair.ab = dev + t->off_ab;
+  t->plan.pair.ba = dev + t->off_ba;
+  t->plan.pair.chirp = t->plan.chirp;
+  t->plan.pair.kern = t->plan.kern;
 }
 
 cudaError_t launch_rows_fwd(const LinePlan& pm, RowIn mode, const void* in, const uint8_t* mask,
                             const float* fest, const float* thresh, float2* out, int N,
                             int nplanes, cudaStream_t st) {
+  if (pm.pair.A) {
+    PairRowArgs q{};
+    q.p = pm.pair; q.in = in; q.mask = mask; q.fest = fest; q.thresh = thresh; q.z = out;
+    q.N = N; q.nplanes = nplanes; q.mode = mode;
+    return launch_pair_rows(0, q, st);
+  }
   RowArgs a{};
   a.pm = pm; a.in = in; a.mask = mask; a.fest = fest; a.thresh = thresh; a.z = out;
   a.N = N; a.nplanes = nplanes; a.C = row_lines(pm); a.pitch = pm.P + 1; a.mode = mode;
@@ -732,6 +863,12 @@ cudaError_t launch_rows_fwd(const LinePlan& pm, RowIn mode, const void* in, cons
 
 cudaError_t launch_rows_inv(const LinePlan& pm, const float2* in, void* out, bool bf16,
                             float scale, int N, int nplanes, cudaStream_t st) {
+  if (pm.pair.A) {
+    PairRowArgs q{};
+    q.p = pm.pair; q.z = const_cast<float2*>(in); q.out = out; q.scale = scale;
+    q.N = N; q.nplanes = nplanes; q.mode = bf16 ? 1 : 0;
+    return launch_pair_rows(1, q, st);
+  }
   RowArgs a{};
   a.pm = pm; a.z = const_cast<float2*>(in); a.out = out; a.scale = scale;
   a.N = N; a.nplanes = nplanes; a.C = row_lines(pm); a.pitch = pm.P + 1; a.mode = bf16 ? 1 : 0;
@@ -741,6 +878,11 @@ cudaError_t launch_rows_inv(const LinePlan& pm, const float2* in, void* out, boo
 
 cudaError_t launch_rows_shrink(const LinePlan& pm, float2* z, const float* thresh, float scale,
                                int N, int nplanes, cudaStream_t st) {
+  if (pm.pair.A) {
+    PairRowArgs q{};
+    q.p = pm.pair; q.z = z; q.thresh = thresh; q.scale = scale; q.N = N; q.nplanes = nplanes;
+    return launch_pair_rows(2, q, st);
+  }
   RowArgs a{};
   a.pm = pm; a.z = z; a.thresh = thresh; a.scale = scale;
   a.N = N; a.nplanes = nplanes; a.C = row_lines(pm); a.pitch = pm.P + 1;
@@ -749,6 +891,11 @@ cudaError_t launch_rows_shrink(const LinePlan& pm, float2* z, const float* thres
 }
 
 cudaError_t launch_cols_fwd(const LinePlan& pn, float2* X, int W, int nplanes, cudaStream_t st) {
+  if (pn.pair.A) {
+    PairColArgs q{};
+    q.p = pn.pair; q.A = X; q.W = W; q.kind = PCOL_FWD;
+    return launch_pair_cols(nplanes, q, st);
+  }
   ColArgs a{};
   a.pn = pn; a.A = X; a.W = W; a.C = col_lines(pn, W); a.pitch = pn.P + 1;
   const size_t smem = 2 * (size_t)a.C * a.pitch * sizeof(float2);
@@ -758,6 +905,12 @@ cudaError_t launch_cols_fwd(const LinePlan& pn, float2* X, int W, int nplanes, c
 cudaError_t launch_cols_dec(const LinePlan& pn, const float2* X, float2* T, const void* G,
                             bool cplx, const float* invW, int W, int K, int s0, int S,
                             cudaStream_t st) {
+  if (pn.pair.A) {
+    PairColArgs q{};
+    q.p = pn.pair; q.X = X; q.T = T; q.G = G; q.cplx = cplx; q.invW = invW;
+    q.W = W; q.K = K; q.s0 = s0; q.S = S; q.kind = PCOL_DEC;
+    return launch_pair_cols(S, q, st);
+  }
   ColArgs a{};
   a.pn = pn; a.X = X; a.T = T; a.G = G; a.cplx = cplx; a.invW = invW;
   a.W = W; a.K = K; a.s0 = s0; a.S = S; a.C = col_lines(pn, W); a.pitch = pn.P + 1;
@@ -772,20 +925,23 @@ cudaError_t launch_cols_rec(const LinePlan& pn, float2* T, float2* A, const void
   a.pn = pn; a.T = T; a.A = A; a.G = G; a.cplx = cplx; a.invW = invW;
   a.W = W; a.K = K; a.s0 = s0; a.S = S; a.C = col_lines(pn, W); a.pitch = pn.P + 1;
   const int nimg = S > 0 ? (s0 + S - 1) / K - s0 / K + 1 : 0;
+  if (pn.pair.A) {
+    PairColArgs q{};
+    q.p = pn.pair; q.T = T; q.A = A; q.G = G; q.cplx = cplx; q.invW = invW;
+    q.W = W; q.K = K; q.s0 = s0; q.S = S;
+    // three CTAs per SM, about four waves, each group at least ceil(K / 16) subbands
+    q.groups = rec_groups((long long)((W + 7) / 8) * nimg, 3, std::min(S, K));
+    q.kind = PCOL_REC;
+    cudaError_t e = launch_pair_cols(nimg, q, st);
+    if (e) return e;
+    q.kind = PCOL_FIN;
+    return launch_pair_cols(nimg, q, st);
+  }
   const size_t smem = 2 * (size_t)a.C * a.pitch * sizeof(float2);
   const size_t smem_rec = 3 * (size_t)a.C * a.pitch * sizeof(float2);   // + the prefetch buffer
   const unsigned cb = (unsigned)((W + a.C - 1) / a.C);
-  // subband groups per image: about four waves of CTAs (smem-bound residency)
-  // with at least ceil(K / 16) subbands a group, so that one image's K
-  // transforms are spread over the GPU instead of running in one CTA
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const long long per_sm = std::max<long long>(1, (228 * 1024) / (long long)(smem_rec + 1024));
-  const long long want = 4LL * std::max(sms, 1) * per_sm;
-  const long long base = std::max<long long>(1, (long long)cb * nimg);
-  a.groups = (int)std::max<long long>(1, std::min<long long>({(want + base - 1) / base, 16,
-                                                              std::min(S, K)}));
+  a.groups = rec_groups((long long)cb * nimg, per_sm, std::min(S, K));
   cudaError_t e = launch(k_cols<COL_REC>, dim3(cb, nimg, a.groups), COL_THREADS, smem_rec, st, a);
   if (e) return e;
   return launch(k_cols<COL_FIN>, dim3(cb, nimg), COL_THREADS, smem, st, a);

@@ -10,7 +10,9 @@
 // every line DFT in shared memory with a mixed-radix Stockham FFT (all prime
 // factors <= 61), or with Bluestein's chirp-z algorithm (a larger prime
 // factor: the length-L DFT becomes a circular convolution of length P = the
-// power of two >= 2L - 1).
+// power of two >= 2L - 1).  Lengths that are products of two small radices, and
+// Bluestein lengths up to 512, run on the two-stage register kernels of
+// general_pairs.cuh.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -26,6 +28,16 @@ constexpr int MAX_LEN = 4096;     // longest side
 constexpr int MAX_STAGES = 16;
 constexpr int MAX_DIRECT_PRIME = 61;
 
+// Lines of the two-stage register kernels (general_pairs.cuh): length L = A B, or
+// Bluestein's P = A B >= 2 L - 1.  A = 0: no pair, the kernels of general.cu.
+struct PairPlan {
+  int L, A, B, bluestein;
+  const float2* ab;          // [(m - 1) A + k] = exp(-2 pi i m k / P), m < B, k < A
+  const float2* ba;          // [(m - 1) B + k], m < A, k < B
+  const float2* chirp;       // [L] exp(-i pi n^2 / L) (Bluestein)
+  const float2* kern;        // [P] DFT_P(h) / P, h[m] = conj chirp[|m|]
+};
+
 // Forward DFT of length L, X[k] = sum_n x[n] exp(-2 pi i n k / L); the
 // inverse is taken as conj(DFT(conj(x))).  Pointers refer to device tables.
 struct LinePlan {
@@ -37,6 +49,7 @@ struct LinePlan {
   const float2* tw;          // [P]  exp(-2 pi i q / P)
   const float2* chirp;       // [L]  exp(-i pi n^2 / L)              (Bluestein)
   const float2* kern;        // [P]  DFT_P(h) / P, h[m] = conj chirp[|m|] (Bluestein)
+  PairPlan pair;
 };
 
 // Host-side tables of one length, computed in float64 and rounded; offsets
@@ -44,7 +57,7 @@ struct LinePlan {
 struct LineTables {
   LinePlan plan{};
   std::vector<float2> data;
-  size_t off_tw = 0, off_chirp = 0, off_kern = 0;
+  size_t off_tw = 0, off_chirp = 0, off_kern = 0, off_ab = 0, off_ba = 0;
 };
 // Builds the plan and tables of length L (1 <= L <= MAX_LEN).
 LineTables make_line_tables(int L);
@@ -70,6 +83,35 @@ cudaError_t launch_rows_inv(const LinePlan& pm, const float2* in, void* out, boo
                             float scale, int N, int nplanes, cudaStream_t st);
 cudaError_t launch_rows_shrink(const LinePlan& pm, float2* z, const float* thresh, float scale,
                                int N, int nplanes, cudaStream_t st);
+
+// The same passes on the two-stage register kernels (plans with pair.A > 0).
+struct PairRowArgs {
+  PairPlan p;                // rows: length M
+  const void* in;            // forward: [nplanes][N][M] reals (f_masked when masked)
+  const uint8_t* mask;       // forward, masked
+  const float* fest;         // forward, masked
+  const float* thresh;       // [nplanes] or null (forward), [nplanes] (shrink)
+  float2* z;                 // half-spectrum planes [nplanes][N][M/2+1]
+  void* out;                 // inverse: float32 / bfloat16 [nplanes][N][M]
+  float scale;               // inverse, shrink
+  int N, nplanes;
+  int mode;                  // forward: RowIn; inverse: 1 = bfloat16 out
+};
+enum PairColKind : int { PCOL_FWD, PCOL_DEC, PCOL_REC, PCOL_FIN };
+struct PairColArgs {
+  PairPlan p;                // columns: length N
+  const float2* X;           // PCOL_DEC: image spectra [B][N][W]
+  float2* T;                 // PCOL_DEC out / PCOL_REC, PCOL_FIN in: staging [S][N][W]
+  float2* A;                 // PCOL_FWD planes (in place) / PCOL_FIN accumulators [B][N][W]
+  const void* G;             // float [K][N][W] or float2 [K][N][W]
+  const float* invW;         // [N][W] or null
+  int W, K, s0, S, cplx;     // W = M/2 + 1 stored columns
+  int groups;                // PCOL_REC, PCOL_FIN: subband groups per image
+  int kind;
+};
+// kind: 0 forward, 1 inverse, 2 shrink.
+cudaError_t launch_pair_rows(int kind, const PairRowArgs& a, cudaStream_t st);
+cudaError_t launch_pair_cols(int planes, const PairColArgs& a, cudaStream_t st);
 
 // Column passes (columns of length N, plan pn) on half-spectrum planes of
 // W = M/2 + 1 columns.
