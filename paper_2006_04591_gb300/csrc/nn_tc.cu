@@ -161,23 +161,46 @@ __device__ __forceinline__ float4 load4(const float* row, int gx, int W) {
   return make_float4(lo.x, lo.y, hi.x, hi.y);
 }
 
+// What a thread loads of every row of one unit: its items' first pixel in row 0
+// and how many of the 8 channels exist (0: nothing to load), so that a row costs an
+// add and 8 loads per item.
 template <int CG>
-__device__ __forceinline__ void conv_load_row(const ConvTcArgs& a, ConvRegs<CG>& R, int b, int gy,
-                                              int x0, int tid) {
+struct ConvSrc {
+  const float* p[ConvRegs<CG>::ITEMS];
+  int gx[ConvRegs<CG>::ITEMS], nch[ConvRegs<CG>::ITEMS];
+};
+template <int CG>
+__device__ __forceinline__ void conv_src(const ConvTcArgs& a, ConvSrc<CG>& s, int b, int x0, int tid) {
   constexpr int PG = PW / 4;
-  const size_t cs = (size_t)a.H * a.W;
-  const bool rok = gy >= 0 && gy < a.H;
 #pragma unroll
   for (int k = 0; k < ConvRegs<CG>::ITEMS; ++k) {
     const int idx = tid + k * CONV_THREADS;
     const int cg = idx / PG, q = idx - cg * PG;
     const int gx = x0 - 4 + 4 * q;
-    const bool ok = rok && idx < CG * PG;
-    const float* row = a.in + (((size_t)b * a.Cin + cg * 8) * a.H + (ok ? gy : 0)) * a.W;
+    const bool ok = idx < CG * PG && cg * 8 < a.Cin && gx + 3 >= 0 && gx < a.W;
+    s.gx[k] = gx;
+    s.nch[k] = ok ? min(8, a.Cin - cg * 8) : 0;
+    s.p[k] = a.in + ((size_t)b * a.Cin + (ok ? cg * 8 : 0)) * a.H * a.W + (ok ? gx : 0);
+  }
+}
+
+template <int CG>
+__device__ __forceinline__ void conv_load_row(const ConvTcArgs& a, const ConvSrc<CG>& s,
+                                              ConvRegs<CG>& R, int gy) {
+  const size_t cs = (size_t)a.H * a.W;
+  const bool rok = gy >= 0 && gy < a.H, vec = (a.W & 3) == 0;
 #pragma unroll
-    for (int c = 0; c < 8; ++c)
-      R.v[k][c] = (ok && cg * 8 + c < a.Cin) ? load4(row + c * cs, gx, a.W)
-                                             : make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int k = 0; k < ConvRegs<CG>::ITEMS; ++k) {
+    const int n = rok ? s.nch[k] : 0;
+    const float* p = s.p[k] + (size_t)(rok ? gy : 0) * a.W;
+    if (vec && n == 8) {         // W a multiple of 4: the group lies wholly inside the row
+#pragma unroll
+      for (int c = 0; c < 8; ++c) R.v[k][c] = __ldg(reinterpret_cast<const float4*>(p + c * cs));
+    } else {
+#pragma unroll
+      for (int c = 0; c < 8; ++c)
+        R.v[k][c] = c < n ? load4(p + c * cs - s.gx[k], s.gx[k], a.W) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
   }
 }
 
@@ -262,17 +285,25 @@ __global__ void __launch_bounds__(CONV_THREADS, (ConvTcT<CG, NP>::MINB)) k_conv3
   const int nunits = a.B * tiles_x * runs;
   uint32_t phase = 0;
   ConvRegs<CG> R;
+  constexpr int HC = NP / 2;
+  const int quarter = warp & 3, n0 = (warp >> 2) * HC;   // this warp's TMEM lanes and columns
+  constexpr int BREG = HC <= 24 ? HC : 1;   // wider tiles have no registers left for the bias
+  float bias[BREG];
+#pragma unroll
+  for (int n = 0; n < BREG; ++n) bias[n] = a.bias && n0 + n < a.Cout ? __ldg(a.bias + n0 + n) : 0.f;
   for (int u = blockIdx.x; u < nunits && !s_fail; u += gridDim.x) {
     const int b = u / (tiles_x * runs), rem = u - b * tiles_x * runs;
     const int xt = rem / runs, y0 = (rem - xt * runs) * RU, y1 = min(a.H, y0 + RU);
     const int x0 = xt * TC_M;
     // the three rows of the first output row (the previous unit's MMAs are
     // done), then the loads of row y0 + 2 start
+    ConvSrc<CG> src;
+    conv_src<CG>(a, src, b, x0, tid);
     for (int gy = y0 - 1; gy <= y0 + 1; ++gy) {
-      conv_load_row<CG>(a, R, b, gy, x0, tid);
+      conv_load_row<CG>(a, src, R, gy);
       conv_store_row<CG>(R, ring + (size_t)((gy + 4) & 3) * P::RBYTES, tid);
     }
-    if (y0 + 1 < y1) conv_load_row<CG>(a, R, b, y0 + 2, x0, tid);
+    if (y0 + 1 < y1) conv_load_row<CG>(a, src, R, y0 + 2);
     for (int y = y0; y < y1; ++y) {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // staged rows -> async proxy
       tc_fence_before();
@@ -304,9 +335,10 @@ __global__ void __launch_bounds__(CONV_THREADS, (ConvTcT<CG, NP>::MINB)) k_conv3
       // no MMA in flight reads; then the loads of row y + 3 start
       if (y + 1 < y1) {
         conv_store_row<CG>(R, ring + (size_t)((y + 2) & 3) * P::RBYTES, tid);
-        if (y + 2 < y1) conv_load_row<CG>(a, R, b, y + 3, x0, tid);
+        if (y + 2 < y1) conv_load_row<CG>(a, src, R, y + 3);
       }
-      if (!mbar_wait(smem_u32(&mbar), phase)) {
+      // one warp polls, the others wait in the barrier
+      if (warp == 0 && !mbar_wait(smem_u32(&mbar), phase)) {
         atomicOr(&g_tc_err, 1u);
         s_fail = 1;
       }
@@ -316,20 +348,19 @@ __global__ void __launch_bounds__(CONV_THREADS, (ConvTcT<CG, NP>::MINB)) k_conv3
       tc_fence_after();
       // warp w reads TMEM lanes 32 (w % 4) .. + 31 (= pixels), columns
       // (w / 4) NP/2 .. + NP/2 - 1 (= output channels)
-      constexpr int HC = NP / 2;
-      const int quarter = warp & 3, n0 = (warp >> 2) * HC;
       uint32_t acc[HC];
 #pragma unroll
       for (int q = 0; q < HC / 8; ++q)
         SHL_TMEM_LD8(acc + 8 * q, tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(n0 + 8 * q));
       asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
       const int px = x0 + quarter * 32 + lane;     // the last tile of a row may be ragged
-      float* o = a.out + (((size_t)b * a.Cout) * a.H + y) * a.W + px;
+      if (px < a.W) {
+        float* o = a.out + (((size_t)b * a.Cout + n0) * a.H + y) * a.W + px;
 #pragma unroll
-      for (int n = 0; n < HC; ++n) {
-        const int ch = n0 + n;
-        if (ch < a.Cout && px < a.W)
-          o[ch * cs] = __uint_as_float(acc[n]) + (a.bias ? __ldg(a.bias + ch) : 0.f);
+        for (int n = 0; n < HC; ++n, o += cs)
+          if (n0 + n < a.Cout)
+            *o = __uint_as_float(acc[n]) +
+                 (BREG == HC ? bias[n % BREG] : a.bias ? __ldg(a.bias + n0 + n) : 0.f);
       }
       tc_fence_before();   // TMEM reads done before the next row's MMAs (barrier at loop top)
     }
@@ -363,7 +394,7 @@ struct WgradTcArgs {
 
 template <int NP>
 struct WgradTcT {
-  static constexpr int THREADS = 256;                       // 8 warps stage, 4 read TMEM
+  static constexpr int THREADS = 512;                       // 16 warps stage, 4 read TMEM
   static constexpr int PG = TC_M / 8;                       // pixel groups per unit row
   static constexpr int SLOTS = 4;                           // input-row ring
   static constexpr size_t ABYTES = (size_t)PG * 128 * 16;   // one input row: [pg][r][8]
@@ -590,7 +621,7 @@ __global__ void __launch_bounds__(WgradTcT<NP>::THREADS, 1) k_wgrad_tc(WgradTcAr
           wgrad_load_gout<NP>(a, R, b, y + 2, x0, tid);
         }
       }
-      if (!mbar_wait(smem_u32(&mbar), phase)) {
+      if (warp == 0 && !mbar_wait(smem_u32(&mbar), phase)) {   // the others wait in the barrier
         atomicOr(&g_tc_err, 1u);
         s_fail = 1;
       }
