@@ -384,12 +384,17 @@ __global__ void __launch_bounds__(CONV_THREADS, (ConvTcT<CG, NP>::MINB)) k_conv3
 // both staged as bfloat16 K-major core matrices [pixel/8][row][8 pixels].
 // A CTA accumulates all its units in TMEM and writes one partial
 // gw[o][i][dy][dx]; k_wgrad_reduce sums the partials in CTA order.
+// 3 Cin <= 128 rows hold at most WGRAD_CH input channels; wider layers run in groups
+// of them, one per blockIdx.y, which write disjoint entries of the same partials (the
+// bias ones come from the first group).
+constexpr int WGRAD_CH = 42;
 struct WgradTcArgs {
-  const float* in;      // [B][Cin][H][W]
+  const float* in;      // [B][Ctot][H][W]
   const float* gout;    // [B][Cout][H][W]
-  float* part;          // [gridDim.x][Cout * Cin * 9 + Cout]: weight then bias partials
-  int B, Cin, Cout, H, W;
+  float* part;          // [gridDim.x][Cout * Ctot * 9 + Cout]: weight then bias partials
+  int B, Ctot, Cout, H, W;
   int rows_per_unit;    // output rows one CTA walks down per unit
+  int Cin;              // channels of this CTA's group (set in the kernel)
 };
 
 template <int NP>
@@ -417,31 +422,57 @@ struct WgradRegs {
   float4 g[WgradTcT<NP>::BITEMS][2];     // gout: pixels x0+8pg .. x0+8pg+7
 };
 
+// Where a thread's items lie in row 0 of the unit's image, and which of their
+// pixels exist (items without any: null), so that a row costs an add and the loads.
 template <int NP>
-__device__ __forceinline__ void wgrad_load_in(const WgradTcArgs& a, WgradRegs<NP>& R, int b, int gy,
-                                              int x0, int tid) {
+struct WgradSrc {
+  const float* in[WgradTcT<NP>::IITEMS];
+  const float* g[WgradTcT<NP>::BITEMS];
+  int ix[WgradTcT<NP>::IITEMS], gx[WgradTcT<NP>::BITEMS];   // first pixel of the group
+  int di[WgradTcT<NP>::IITEMS], dg[WgradTcT<NP>::BITEMS];   // byte offsets in the staged rows
+};
+template <int NP>
+__device__ __forceinline__ void wgrad_src(const WgradTcArgs& a, WgradSrc<NP>& s, int b, int x0, int tid) {
   using P = WgradTcT<NP>;
-  const bool rok = gy >= 0 && gy < a.H;
 #pragma unroll
   for (int k = 0; k < P::IITEMS; ++k) {
-    const int idx = tid + k * P::THREADS;
+    const int idx = tid + k * P::THREADS, pg = idx / a.Cin, i = idx - pg * a.Cin;
+    s.ix[k] = x0 + 8 * pg;
+    s.di[k] = (pg * 128 + i) * 16;
+    s.in[k] = pg < P::PG ? a.in + ((size_t)b * a.Ctot + i) * a.H * a.W + s.ix[k] : nullptr;
+  }
+#pragma unroll
+  for (int k = 0; k < P::BITEMS; ++k) {
+    const int idx = tid + k * P::THREADS, pg = idx / a.Cout, o = idx - pg * a.Cout;
+    s.gx[k] = x0 + 8 * pg;
+    s.dg[k] = (pg * NP + o) * 16;
+    s.g[k] = pg < P::PG ? a.gout + ((size_t)b * a.Cout + o) * a.H * a.W + s.gx[k] : nullptr;
+  }
+}
+
+template <int NP>
+__device__ __forceinline__ void wgrad_load_in(const WgradTcArgs& a, const WgradSrc<NP>& s,
+                                              WgradRegs<NP>& R, int gy) {
+  using P = WgradTcT<NP>;
+  const bool rok = gy >= 0 && gy < a.H, vec = (a.W & 3) == 0;
+#pragma unroll
+  for (int k = 0; k < P::IITEMS; ++k) {
     float* e = R.e[k];
-    if (rok && idx < a.Cin * P::PG) {
-      const int pg = idx / a.Cin, i = idx - pg * a.Cin;
-      const int xs = x0 + 8 * pg;
-      const float* row = a.in + (((size_t)b * a.Cin + i) * a.H + gy) * a.W;
-      if ((a.W & 3) == 0 && xs + 8 <= a.W) {
-        const float4 v0 = __ldg(reinterpret_cast<const float4*>(row + xs));
-        const float4 v1 = __ldg(reinterpret_cast<const float4*>(row + xs + 4));
-        e[0] = xs > 0 ? __ldg(row + xs - 1) : 0.f;
+    if (rok && s.in[k]) {
+      const int xs = s.ix[k];
+      const float* p = s.in[k] + (size_t)gy * a.W;
+      if (vec && xs + 8 <= a.W) {
+        const float4 v0 = __ldg(reinterpret_cast<const float4*>(p));
+        const float4 v1 = __ldg(reinterpret_cast<const float4*>(p + 4));
+        e[0] = xs > 0 ? __ldg(p - 1) : 0.f;
         e[1] = v0.x; e[2] = v0.y; e[3] = v0.z; e[4] = v0.w;
         e[5] = v1.x; e[6] = v1.y; e[7] = v1.z; e[8] = v1.w;
-        e[9] = xs + 8 < a.W ? __ldg(row + xs + 8) : 0.f;
+        e[9] = xs + 8 < a.W ? __ldg(p + 8) : 0.f;
       } else {                       // ragged last tile, or rows not 16-byte aligned
 #pragma unroll
         for (int j = 0; j < 10; ++j) {
           const int x = xs - 1 + j;
-          e[j] = x >= 0 && x < a.W ? __ldg(row + x) : 0.f;
+          e[j] = x >= 0 && x < a.W ? __ldg(p + j - 1) : 0.f;
         }
       }
     } else {
@@ -453,19 +484,17 @@ __device__ __forceinline__ void wgrad_load_in(const WgradTcArgs& a, WgradRegs<NP
 
 // -> the three shifted copies A[r = dx * Cin + i][p] = in[i][gy][x0 + p + dx - 1]
 template <int NP>
-__device__ __forceinline__ void wgrad_store_in(const WgradTcArgs& a, const WgradRegs<NP>& R,
-                                               uint8_t* dst, int tid) {
+__device__ __forceinline__ void wgrad_store_in(const WgradTcArgs& a, const WgradSrc<NP>& s,
+                                               const WgradRegs<NP>& R, uint8_t* dst) {
   using P = WgradTcT<NP>;
 #pragma unroll
   for (int k = 0; k < P::IITEMS; ++k) {
-    const int idx = tid + k * P::THREADS;
-    if (idx < a.Cin * P::PG) {
-      const int pg = idx / a.Cin, i = idx - pg * a.Cin;
+    if (s.in[k]) {
       const float* e = R.e[k];
-      uint8_t* d = dst + ((size_t)pg * 128 + i) * 16;
+      uint8_t* d = dst + s.di[k];
 #pragma unroll
       for (int dx = 0; dx < 3; ++dx)   // pixel x0+8pg+j-1+dx = e[j + dx]
-        *reinterpret_cast<uint4*>(d + (size_t)dx * a.Cin * 16) =
+        *reinterpret_cast<uint4*>(d + dx * a.Cin * 16) =
             make_uint4(pack_bf16(e[dx], e[dx + 1]), pack_bf16(e[dx + 2], e[dx + 3]),
                        pack_bf16(e[dx + 4], e[dx + 5]), pack_bf16(e[dx + 6], e[dx + 7]));
     }
@@ -473,23 +502,22 @@ __device__ __forceinline__ void wgrad_store_in(const WgradTcArgs& a, const Wgrad
 }
 
 template <int NP>
-__device__ __forceinline__ void wgrad_load_gout(const WgradTcArgs& a, WgradRegs<NP>& R, int b,
-                                                int y, int x0, int tid) {
+__device__ __forceinline__ void wgrad_load_gout(const WgradTcArgs& a, const WgradSrc<NP>& s,
+                                                WgradRegs<NP>& R, int y) {
   using P = WgradTcT<NP>;
+  const bool vec = (a.W & 3) == 0;
 #pragma unroll
   for (int k = 0; k < P::BITEMS; ++k) {
-    const int idx = tid + k * P::THREADS;
-    if (idx < a.Cout * P::PG) {
-      const int pg = idx / a.Cout, o = idx - pg * a.Cout;
-      const int xs = x0 + 8 * pg;
-      const float* row = a.gout + (((size_t)b * a.Cout + o) * a.H + y) * a.W;
-      if ((a.W & 3) == 0 && xs + 8 <= a.W) {
-        R.g[k][0] = __ldg(reinterpret_cast<const float4*>(row + xs));
-        R.g[k][1] = __ldg(reinterpret_cast<const float4*>(row + xs + 4));
+    if (s.g[k]) {
+      const int xs = s.gx[k];
+      const float* p = s.g[k] + (size_t)y * a.W;
+      if (vec && xs + 8 <= a.W) {
+        R.g[k][0] = __ldg(reinterpret_cast<const float4*>(p));
+        R.g[k][1] = __ldg(reinterpret_cast<const float4*>(p + 4));
       } else {                       // ragged last tile, or rows not 16-byte aligned
         float v[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) v[j] = xs + j < a.W ? __ldg(row + xs + j) : 0.f;
+        for (int j = 0; j < 8; ++j) v[j] = xs + j < a.W ? __ldg(p + j) : 0.f;
         R.g[k][0] = make_float4(v[0], v[1], v[2], v[3]);
         R.g[k][1] = make_float4(v[4], v[5], v[6], v[7]);
       }
@@ -500,18 +528,15 @@ __device__ __forceinline__ void wgrad_load_gout(const WgradTcArgs& a, WgradRegs<
 // -> B[o][p] = gout[o][y][x0 + p]; bsum[k] gathers this thread's float32
 // bias partial (item k always has channel (tid + k THREADS) mod Cout)
 template <int NP>
-__device__ __forceinline__ void wgrad_store_gout(const WgradTcArgs& a, const WgradRegs<NP>& R,
-                                                 uint8_t* dst, int tid,
-                                                 float (&bsum)[WgradTcT<NP>::BITEMS]) {
+__device__ __forceinline__ void wgrad_store_gout(const WgradSrc<NP>& s, const WgradRegs<NP>& R,
+                                                 uint8_t* dst, float (&bsum)[WgradTcT<NP>::BITEMS]) {
   using P = WgradTcT<NP>;
 #pragma unroll
   for (int k = 0; k < P::BITEMS; ++k) {
-    const int idx = tid + k * P::THREADS;
-    if (idx < a.Cout * P::PG) {
-      const int pg = idx / a.Cout, o = idx - pg * a.Cout;
+    if (s.g[k]) {
       const float4 v0 = R.g[k][0], v1 = R.g[k][1];
       bsum[k] += ((v0.x + v0.y) + (v0.z + v0.w)) + ((v1.x + v1.y) + (v1.z + v1.w));
-      *reinterpret_cast<uint4*>(dst + ((size_t)pg * NP + o) * 16) =
+      *reinterpret_cast<uint4*>(dst + s.dg[k]) =
           make_uint4(pack_bf16(v0.x, v0.y), pack_bf16(v0.z, v0.w), pack_bf16(v1.x, v1.y),
                      pack_bf16(v1.z, v1.w));
     }
@@ -523,9 +548,13 @@ __device__ __forceinline__ void wgrad_store_gout(const WgradTcArgs& a, const Wgr
 // (row y + 2 staged while the MMAs of row y run), gout rows double-buffered;
 // every MMA of the launch accumulates into the same three TMEM tiles.
 template <int NP>
-__global__ void __launch_bounds__(WgradTcT<NP>::THREADS, 1) k_wgrad_tc(WgradTcArgs a) {
+__global__ void __launch_bounds__(WgradTcT<NP>::THREADS, 1) k_wgrad_tc(const WgradTcArgs args) {
   using P = WgradTcT<NP>;
   extern __shared__ __align__(128) uint8_t sm[];
+  const int c0 = blockIdx.y * WGRAD_CH;       // the group's first input channel
+  WgradTcArgs a = args;
+  a.Cin = min(WGRAD_CH, args.Ctot - c0);
+  a.in += (size_t)c0 * a.H * a.W;
   uint8_t* As = sm;                           // SLOTS x [pg][128][8]
   uint8_t* Bs = sm + P::SLOTS * P::ABYTES;    // 2 x [pg][NP][8]
   __shared__ __align__(8) uint64_t mbar;
@@ -571,15 +600,17 @@ __global__ void __launch_bounds__(WgradTcT<NP>::THREADS, 1) k_wgrad_tc(WgradTcAr
     const int x0 = xt * TC_M;
     // the previous unit's MMAs are done: stage rows y0-1..y0+1 and gout row
     // y0, then start the loads of input row y0+2 and gout row y0+1
+    WgradSrc<NP> src;
+    wgrad_src<NP>(a, src, b, x0, tid);
     for (int gy = y0 - 1; gy <= y0 + 1; ++gy) {
-      wgrad_load_in<NP>(a, R, b, gy, x0, tid);
-      wgrad_store_in<NP>(a, R, As + (size_t)((gy + 4) & 3) * P::ABYTES, tid);
+      wgrad_load_in<NP>(a, src, R, gy);
+      wgrad_store_in<NP>(a, src, R, As + (size_t)((gy + 4) & 3) * P::ABYTES);
     }
-    wgrad_load_gout<NP>(a, R, b, y0, x0, tid);
-    wgrad_store_gout<NP>(a, R, Bs + (size_t)(y0 & 1) * P::BBYTES, tid, bsum);
+    wgrad_load_gout<NP>(a, src, R, y0);
+    wgrad_store_gout<NP>(src, R, Bs + (size_t)(y0 & 1) * P::BBYTES, bsum);
     if (y0 + 1 < y1) {
-      wgrad_load_in<NP>(a, R, b, y0 + 2, x0, tid);
-      wgrad_load_gout<NP>(a, R, b, y0 + 1, x0, tid);
+      wgrad_load_in<NP>(a, src, R, y0 + 2);
+      wgrad_load_gout<NP>(a, src, R, y0 + 1);
     }
     for (int y = y0; y < y1; ++y) {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -614,11 +645,11 @@ __global__ void __launch_bounds__(WgradTcT<NP>::THREADS, 1) k_wgrad_tc(WgradTcAr
       // input row y + 2 to the slot of row y - 2, gout row y + 1 to the other
       // B buffer (row y - 1's); then the loads of the rows after them start
       if (y + 1 < y1) {
-        wgrad_store_in<NP>(a, R, As + (size_t)((y + 2) & 3) * P::ABYTES, tid);
-        wgrad_store_gout<NP>(a, R, Bs + (size_t)((y + 1) & 1) * P::BBYTES, tid, bsum);
+        wgrad_store_in<NP>(a, src, R, As + (size_t)((y + 2) & 3) * P::ABYTES);
+        wgrad_store_gout<NP>(src, R, Bs + (size_t)((y + 1) & 1) * P::BBYTES, bsum);
         if (y + 2 < y1) {
-          wgrad_load_in<NP>(a, R, b, y + 3, x0, tid);
-          wgrad_load_gout<NP>(a, R, b, y + 2, x0, tid);
+          wgrad_load_in<NP>(a, src, R, y + 3);
+          wgrad_load_gout<NP>(a, src, R, y + 2);
         }
       }
       if (warp == 0 && !mbar_wait(smem_u32(&mbar), phase)) {   // the others wait in the barrier
@@ -641,11 +672,11 @@ __global__ void __launch_bounds__(WgradTcT<NP>::THREADS, 1) k_wgrad_tc(WgradTcAr
     if (idx < a.Cout * P::PG) bred[idx] = bsum[k];
   }
   __syncthreads();
-  const size_t stride = (size_t)a.Cout * a.Cin * 9 + a.Cout;
-  if (tid < a.Cout) {   // items of channel o: idx = pg * Cout + o
+  const size_t stride = (size_t)a.Cout * a.Ctot * 9 + a.Cout;
+  if (c0 == 0 && tid < a.Cout) {   // items of channel o: idx = pg * Cout + o
     float s = 0.f;
     for (int pg = 0; pg < P::PG; ++pg) s += bred[pg * a.Cout + tid];
-    a.part[(size_t)blockIdx.x * stride + (size_t)a.Cout * a.Cin * 9 + tid] = s;
+    a.part[(size_t)blockIdx.x * stride + (size_t)a.Cout * a.Ctot * 9 + tid] = s;
   }
   // epilogue (warps 0-3): lane r = dx * Cin + i, columns dy * NP + o
   if (!s_fail && warp < 4) {
@@ -665,7 +696,7 @@ __global__ void __launch_bounds__(WgradTcT<NP>::THREADS, 1) k_wgrad_tc(WgradTcAr
           for (int j = 0; j < 16; ++j) {
             const int o = 16 * q + j;
             if (o < a.Cout)
-              part[(((size_t)o * a.Cin + i) * 3 + dy) * 3 + dx] =
+              part[(((size_t)o * a.Ctot + c0 + i) * 3 + dy) * 3 + dx] =
                   blockIdx.x < nunits ? __uint_as_float(acc[j]) : 0.f;
           }
         }
@@ -689,7 +720,8 @@ __global__ void k_wgrad_reduce(const float* __restrict__ part, float* __restrict
   const int n = nw + nb;
   if (e >= n) return;
   float s = 0.f;
-  for (int c = 0; c < nparts; ++c) s += part[(size_t)c * n + e];
+#pragma unroll 8
+  for (int c = 0; c < nparts; ++c) s += part[(size_t)c * n + e];   // eight loads in flight
   if (e < nw) gw[e] = s;
   else if (gb) gb[e - nw] = s;
 }
@@ -716,7 +748,7 @@ cudaError_t launch_wgrad(const WgradTcArgs& a, int grid, cudaStream_t st) {
   auto k = k_wgrad_tc<NP>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P::SMEM);
   if (e) return e;
-  k<<<grid, P::THREADS, P::SMEM, st>>>(a);
+  k<<<dim3(grid, (a.Ctot + WGRAD_CH - 1) / WGRAD_CH), P::THREADS, P::SMEM, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -1139,6 +1171,29 @@ size_t shl_nn_conv3x3_backward_weight_tc_workspace_floats(int B, int Ci, int Co,
   return (size_t)grid * ((size_t)Co * Ci * 9 + Co);
 }
 
+static shl_status wgrad_run(const float* in, const float* gout, float* gw, float* gb, int B, int Ci,
+                            int Co, int H, int W, float* ws, void* stream) {
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  int grid = 0, ru = 0;
+  wgrad_plan(B, H, W, &grid, &ru);
+  const WgradTcArgs a{in, gout, ws, B, Ci, Co, H, W, ru, 0};
+  const int np = round16(Co);          // 49..96 output channels: the 96-wide tile
+  cudaError_t e = np == 16 ? launch_wgrad<16>(a, grid, st)
+                : np == 32 ? launch_wgrad<32>(a, grid, st)
+                : np == 48 ? launch_wgrad<48>(a, grid, st)
+                           : launch_wgrad<96>(a, grid, st);
+  if (e == cudaSuccess) {
+    const int nw = Co * Ci * 9;
+    k_wgrad_reduce<<<(nw + Co + 127) / 128, 128, 0, st>>>(ws, gw, gb, grid, nw, Co);
+    e = cudaGetLastError();
+  }
+  if (e != cudaSuccess) {
+    g_tc_msg = "conv3x3_backward_weight_tc: launch failed";
+    return SHL_ECUDA;
+  }
+  return SHL_OK;
+}
+
 shl_status shl_nn_conv3x3_backward_weight_tc(const float* in, const float* gout, float* gw,
                                              float* gb, int B, int Ci, int Co, int H, int W,
                                              float* ws, void* stream) {
@@ -1147,25 +1202,28 @@ shl_status shl_nn_conv3x3_backward_weight_tc(const float* in, const float* gout,
     g_tc_msg = "conv3x3_backward_weight_tc: bad arguments, unsupported shape or misaligned input";
     return SHL_EINVAL;
   }
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  return wgrad_run(in, gout, gw, gb, B, Ci, Co, H, W, ws, stream);
+}
+
+size_t shl_nn_conv3x3_backward_weight_tc_wide_workspace_floats(int B, int Ci, int Co, int H, int W) {
+  if (B < 1 || Ci < 1 || Ci > 4096 ||
+      !shl_nn_conv3x3_wgrad_tc_supported(std::min(Ci, WGRAD_CH), Co, H, W))
+    return 0;
   int grid = 0, ru = 0;
   wgrad_plan(B, H, W, &grid, &ru);
-  const WgradTcArgs a{in, gout, ws, B, Ci, Co, H, W, ru};
-  const int np = round16(Co);          // 49..96 output channels: the 96-wide tile
-  cudaError_t e = np == 16 ? launch_wgrad<16>(a, grid, st)
-                : np == 32 ? launch_wgrad<32>(a, grid, st)
-                : np == 48 ? launch_wgrad<48>(a, grid, st)
-                           : launch_wgrad<96>(a, grid, st);
-  if (e == cudaSuccess) {
-    const int nw = Co * Ci * 9;
-    k_wgrad_reduce<<<(nw + Co + 255) / 256, 256, 0, st>>>(ws, gw, gb, grid, nw, Co);
-    e = cudaGetLastError();
+  return (size_t)grid * ((size_t)Co * Ci * 9 + Co);
+}
+
+shl_status shl_nn_conv3x3_backward_weight_tc_wide(const float* in, const float* gout, float* gw,
+                                                  float* gb, int B, int Ci, int Co, int H, int W,
+                                                  float* ws, void* stream) {
+  if (!in || !gout || !gw || !ws ||
+      shl_nn_conv3x3_backward_weight_tc_wide_workspace_floats(B, Ci, Co, H, W) == 0 ||
+      ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(gout)) & 15u)) {
+    g_tc_msg = "conv3x3_backward_weight_tc_wide: bad arguments, unsupported shape or misaligned input";
+    return SHL_EINVAL;
   }
-  if (e != cudaSuccess) {
-    g_tc_msg = "conv3x3_backward_weight_tc: launch failed";
-    return SHL_ECUDA;
-  }
-  return SHL_OK;
+  return wgrad_run(in, gout, gw, gb, B, Ci, Co, H, W, ws, stream);
 }
 
 shl_status shl_nn_tc_status(void* stream) {

@@ -48,6 +48,8 @@ def lib():
             "shl_nn_conv3x3_wgrad_tc_supported": (i, [i, i, i, i]),
             "shl_nn_conv3x3_backward_weight_tc_workspace_floats": (sz, [i, i, i, i, i]),
             "shl_nn_conv3x3_backward_weight_tc": (i, [vp, vp, vp, vp, i, i, i, i, i, vp, vp]),
+            "shl_nn_conv3x3_backward_weight_tc_wide_workspace_floats": (sz, [i, i, i, i, i]),
+            "shl_nn_conv3x3_backward_weight_tc_wide": (i, [vp, vp, vp, vp, i, i, i, i, i, vp, vp]),
             "shl_nn_tc_last_error": (ctypes.c_char_p, []),
             "shl_nn_prelu_forward": (i, [vp, vp, vp, ll, vp]),
             "shl_nn_reduce_workspace_floats": (sz, [ll]),
@@ -137,6 +139,15 @@ def shl_nn_conv3x3_backward_weight_tc(x, gout, gw, gb):
         _p(x), _p(gout), _p(gw), _p(gb), B, Ci, Co, H, W, _p(ws), _st(x)))
 
 
+def shl_nn_conv3x3_backward_weight_tc_wide(x, gout, gw, gb):
+    B, Ci, H, W = x.shape
+    Co = gout.shape[1]
+    L = lib()
+    ws = _ws(L.shl_nn_conv3x3_backward_weight_tc_wide_workspace_floats(B, Ci, Co, H, W), x)
+    _chk_tc("conv3x3_backward_weight_tc_wide", L.shl_nn_conv3x3_backward_weight_tc_wide(
+        _p(x), _p(gout), _p(gw), _p(gb), B, Ci, Co, H, W, _p(ws), _st(x)))
+
+
 def shl_nn_tc_status(stream=None):
     s = ctypes.c_void_p(None if stream is None else stream.cuda_stream)
     _chk_tc("tc_status", lib().shl_nn_tc_status(s))
@@ -151,15 +162,8 @@ def shl_nn_conv3x3_backward(x, w, gout, need_gin=True, tc=False, tc_w=False):
     if tc_w and Ci <= TC_WCH:
         shl_nn_conv3x3_backward_weight_tc(x, gout, gw, gb)
     elif tc_w:
-        # one call stages at most 42 input channels (3 Ci <= 128 rows); the
-        # weight gradient of an input-channel group depends on that group only
-        for k, (c0, c1) in enumerate(_groups(Ci, TC_WCH)):
-            gwg = torch.empty((Co, c1 - c0, 3, 3), dtype=torch.float32, device=x.device)
-            gbg = torch.empty(Co, dtype=torch.float32, device=x.device)
-            shl_nn_conv3x3_backward_weight_tc(x[:, c0:c1].contiguous(), gout, gwg, gbg)
-            gw[:, c0:c1] = gwg
-            if k == 0:
-                gb.copy_(gbg)
+        xa = x if x.data_ptr() % 16 == 0 else x.clone()   # a view may start anywhere
+        shl_nn_conv3x3_backward_weight_tc_wide(xa, gout, gw, gb)
     ws = _ws(L.shl_nn_conv3x3_workspace_floats(B, Ci, Co, H, W), x) if (not tc_w or
                                                                       (need_gin and not tc)) else None
     if not tc_w and Ci <= 64:
