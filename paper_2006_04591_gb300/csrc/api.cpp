@@ -560,7 +560,7 @@ shl_status reconstruct_impl(const shl_bank* b, const void* coeffs, shl_dtype dty
                                  thresh != nullptr,
                                  static_cast<const char*>(coeffs) + (size_t)s0 * N * M * esz,
                                  nullptr, nullptr, thresh ? thresh + s0 : nullptr, Z, N, Sc,
-                                 b->dTw, st);
+                                 b->dTw, st, true);
     }
     if (e) return cuda_fail(e, "rows_r2c_coeffs");
     {

@@ -89,12 +89,12 @@ __device__ __forceinline__ void dft_prime(float2 (&v)[R]) {
   float2 s[H], d[H];
 #pragma unroll
   for (int m = 1; m <= H; ++m) {
-    s[m - 1] = cadd(v[m], v[R - m]);
-    d[m - 1] = csub(v[m], v[R - m]);
+    s[m - 1] = caddp(v[m], v[R - m]);
+    d[m - 1] = csubp(v[m], v[R - m]);
   }
   const float2 v0 = v[0];
 #pragma unroll
-  for (int m = 0; m < H; ++m) v[0] = cadd(v[0], s[m]);
+  for (int m = 0; m < H; ++m) v[0] = caddp(v[0], s[m]);
   static_for<1, H + 1>([&](auto qi) {
     constexpr int q = decltype(qi)::value;
     float2 a = v0, b = make_float2(0.f, 0.f);
@@ -146,7 +146,7 @@ __device__ __forceinline__ void dft_split(float2 (&v)[R]) {
 template <int R>
 __device__ __forceinline__ void dft_n(float2 (&v)[R]) {
   if constexpr (R == 1) return;
-  else if constexpr (R == 2 || R == 4 || R == 8) dft_reg<R, -1>(v);
+  else if constexpr (R == 2 || R == 4 || R == 8) dft_reg<R, -1, true>(v);
   else if constexpr (pow2_part(R) == R) dft_split<R, 4>(v);
   else if constexpr (is_prime(R)) dft_prime<R>(v);
   else dft_split<R, split_factor(R)>(v);

@@ -231,7 +231,7 @@ __device__ __forceinline__ void r2c_issue(const RowsTArgs& a, char* stage, int t
 // complex) of row r -> R2C (line FFT and conjugate-pair split) -> the
 // transposed tile in shared memory -> out[kx * N + row] for the TR rows.
 // Ends with a CTA barrier, after which the line and tile buffers are free.
-template <int LOG_M>
+template <int LOG_M, bool PK>
 __device__ __forceinline__ void r2c_tile_finish(float2 (&v)[RowsT<LOG_M>::R], float2* line,
                                                 float2* tile, const float2* twl, const float2* ptw,
                                                 float2* out, int N, int r, int j, bool valid,
@@ -239,7 +239,7 @@ __device__ __forceinline__ void r2c_tile_finish(float2 (&v)[RowsT<LOG_M>::R], fl
   using P = RowsT<LOG_M>;
   constexpr int T = P::T, R = P::R, L = P::L, Mh = P::Mh, TR = P::TR, TP = P::TP;
   const float2* twb = ptw + L;                             // lane bases after the split factors
-  line_fft_any<L, R, -1>(v, line, j, 1 + r, twl, twb);
+  line_fft_any<L, R, -1, PK>(v, line, j, 1 + r, twl, twb);
 
   // conjugate-pair split needs Z[L - k]: publish the natural-order line
   group_sync<T>(1 + r);
@@ -272,7 +272,14 @@ __device__ __forceinline__ void r2c_tile_finish(float2 (&v)[RowsT<LOG_M>::R], fl
   __syncthreads();
 }
 
-template <int LOG_M, int INM, bool THRESH>
+// Coefficient rows use packed additions up to M = 512 (R2C 294 -> 284 us, C2R 268 ->
+// 262 us at 16 x 512^2, K = 49); at 1024 they cost (763 -> 780 us at 8 x 1024^2).
+template <int LOG_M>
+__host__ __device__ constexpr bool rows_packed() { return LOG_M < 10; }
+
+// PK: packed additions (coefficient rows; the image's rows feed the bfloat16
+// decomposition as well and keep the scalar form).
+template <int LOG_M, int INM, bool THRESH, bool PK>
 __global__ void __launch_bounds__(RowsT<LOG_M>::THREADS, (r2c_minb<LOG_M, INM>())) k_rows_r2c_t(RowsTArgs a) {
   using P = RowsT<LOG_M>;
   constexpr int T = P::T, R = P::R, L = P::L, Mh = P::Mh, M = P::M;
@@ -389,7 +396,7 @@ __global__ void __launch_bounds__(RowsT<LOG_M>::THREADS, (r2c_minb<LOG_M, INM>()
       }
     }
 
-    r2c_tile_finish<LOG_M>(v, line, tile, twl, ptw, a.out + (size_t)s * Mh * a.N + y0, a.N, r, j,
+    r2c_tile_finish<LOG_M, PK>(v, line, tile, twl, ptw, a.out + (size_t)s * Mh * a.N + y0, a.N, r, j,
                            valid, tid, tile_ok);    // ends with a barrier: tile and stage reusable
   }
 }
@@ -459,14 +466,14 @@ __device__ __forceinline__ void c2r_tile_load(const float2* tile, const float2* 
   }
 }
 
-template <int LOG_M, bool S16 = false>
+template <int LOG_M, bool S16, bool PK>
 __device__ __forceinline__ void c2r_tile_compute(const float2* tile, float2* line,
                                                  const float2* twl, const float2* ptw, int r,
                                                  int j, bool valid,
                                                  float2 (&v)[RowsT<LOG_M>::R]) {
   using P = RowsT<LOG_M>;
   c2r_tile_load<LOG_M, S16>(tile, ptw, r, j, valid, v);
-  line_fft_any<P::L, P::R, +1>(v, line, j, 1 + r, twl, ptw + P::L);
+  line_fft_any<P::L, P::R, +1, PK>(v, line, j, 1 + r, twl, ptw + P::L);
 }
 
 // Row r of the inverse FFT's output v to out + base (float32 or bfloat16).
@@ -495,7 +502,7 @@ __device__ __forceinline__ void c2r_tile_body(const float2* tile, float2* line,
   using P = RowsT<LOG_M>;
   constexpr int T = P::T, R = P::R;
   float2 v[R];
-  c2r_tile_compute<LOG_M, S16>(tile, line, twl, ptw, r, j, valid, v);
+  c2r_tile_compute<LOG_M, S16, (!BF16OUT && rows_packed<LOG_M>())>(tile, line, twl, ptw, r, j, valid, v);
   if (valid) {
 #pragma unroll
     for (int u = 0; u < R; ++u) {
@@ -562,7 +569,7 @@ __global__ void __launch_bounds__(RowsT<LOG_M>::THREADS, (c2r_occ3<LOG_M, S16>()
       __syncthreads();                     // the stage is read: refill it with the next tile
       if (t + (int)gridDim.x < ntiles) c2r_issue<LOG_M, S16>(a, stages, t + gridDim.x, tid);
       cp_async_commit();
-      line_fft_any<L, R, +1>(v, line, j, 1 + r, twl, ptw + L);
+      line_fft_any<L, R, +1, (!BF16OUT && rows_packed<LOG_M>())>(v, line, j, 1 + r, twl, ptw + L);
       if (valid && SHL_IN((size_t)s * a.N + y0 + rr, (size_t)a.nsub * a.N, CHK_C2R_OUT))
         c2r_store_row<LOG_M, BF16OUT>(v, a.out, ((size_t)s * a.N + y0 + rr) * P::M, j);
       continue;
@@ -629,7 +636,7 @@ k_rows_shrink_t(RowsShrinkArgs a) {
     __syncthreads();
     const int s = t / tiles_per_sub, y0 = (t % tiles_per_sub) * TR;
     float2 v[R];
-    c2r_tile_compute<LOG_M>(stages + (k % NST) * SW, line, twl, ptw, r, j, valid, v);
+    c2r_tile_compute<LOG_M, false, rows_packed<LOG_M>()>(stages + (k % NST) * SW, line, twl, ptw, r, j, valid, v);
     const float tau = SHL_IN(s, a.nsub, CHK_SHRINK) ? __ldg(a.thresh + s) : 0.f;
 #pragma unroll
     for (int u = 0; u < R; ++u) {
@@ -638,7 +645,7 @@ k_rows_shrink_t(RowsShrinkArgs a) {
     }
     // the forward line FFT reuses the group's own line buffer after a group
     // sync; the CTA-wide tile reuse is fenced inside r2c_tile_finish
-    r2c_tile_finish<LOG_M>(v, line, work, twl, ptw, a.z + (size_t)s * Mh * a.N + y0, a.N, r, j,
+    r2c_tile_finish<LOG_M, rows_packed<LOG_M>()>(v, line, work, twl, ptw, a.z + (size_t)s * Mh * a.N + y0, a.N, r, j,
                            valid, tid);    // ends with a barrier: tile and stage reusable
   }
   cp_async_wait0();
@@ -649,10 +656,13 @@ k_rows_shrink_t(RowsShrinkArgs a) {
 // instead of two, measured slower at 512 x 512: 0.554 / 0.662 ms against
 // 0.534 / 0.571 ms for decomposition / reconstruction of 16 images; the
 // extra registers leave one CTA per SM.)
-template <int LOG_N>
+// The reconstruction also keeps its sums: 1024-point lines there go as 16 x 16 x 4
+// over 64 lanes (two CTAs per SM instead of one: 569 -> 503 us at 8 x 1024^2,
+// K = 49; the decomposition's and the image's lines are faster as 32 x 32).
+template <int LOG_N, bool REC = false>
 struct LinesT {
   static constexpr int N = 1 << LOG_N;
-  static constexpr int R = LineRadix<N>::R;
+  static constexpr int R = REC && N == 1024 ? 16 : LineRadix<N>::R;
   using C = LineCfg<N, R>;
   static constexpr int T = C::T;
   static constexpr int THREADS = 256;
@@ -713,6 +723,32 @@ __device__ __forceinline__ void dec_group(const float2* X, void* out, const floa
   using P = LinesT<LOG_N>;
   constexpr int T = P::T, R = P::R, N = P::N;
   const float* W = invW ? invW + (size_t)kx * N : nullptr;
+  if constexpr (R >= 32 && !S16) {
+    // 32 values per lane: reading the spectrum line again for every filter (from L2)
+    // leaves two CTAs per SM where holding it left one (4 x 1024^2: 249 -> 215 us;
+    // at 16 values per lane a third CTA gains nothing; the bfloat16 form keeps its
+    // rounding, see dft_reg)
+    for (int sl = sl0; sl < sl1; ++sl) {
+      const int s = s0 + sl, b = s / K, i = s - b * K;
+      const float2* Xp = X + ((size_t)b * Mh + kx) * N;
+      const float* G = Gall + ((size_t)i * Mh + kx) * N;
+      const bool ok = SHL_IN((size_t)b * Mh + kx, (size_t)nimg * Mh, CHK_DEC_X) &&
+                      SHL_IN((size_t)i * Mh + kx, (size_t)K * Mh, CHK_DEC_G);
+      float2 v[R];
+#pragma unroll
+      for (int u = 0; u < R; ++u) {
+        float gv = ok ? __ldg(G + j + u * T) * scale : 0.f;
+        if (W) gv *= __ldg(W + j + u * T);
+        v[u] = ok ? cscale(Xp[j + u * T], gv) : make_float2(0.f, 0.f);
+      }
+      line_fft_any<N, R, +1, !S16>(v, line, j, 1 + g, twl, twl + LineTw<N, R>::WORDS);
+      if (!SHL_IN((size_t)sl * Mh + kx, (size_t)nstage * Mh, CHK_DEC_OUT)) continue;
+      float2* o = static_cast<float2*>(out) + ((size_t)sl * Mh + kx) * N;
+#pragma unroll
+      for (int u = 0; u < R; ++u) o[j + u * T] = v[u];
+    }
+    return;
+  }
   float2 Xl[R];
   float gn[R];
   int b_loaded = -1;
@@ -749,7 +785,7 @@ __device__ __forceinline__ void dec_group(const float2* X, void* out, const floa
       if (W) gv *= __ldg(W + j + u * T);
       v[u] = cscale(Xl[u], gv);
     }
-    line_fft_any<N, R, +1>(v, line, j, 1 + g, twl, twl + LineTw<N, R>::WORDS);
+    line_fft_any<N, R, +1, !S16>(v, line, j, 1 + g, twl, twl + LineTw<N, R>::WORDS);
     if (SHL_IN((size_t)sl * Mh + kx, (size_t)nstage * Mh, CHK_DEC_OUT)) {
       if constexpr (S16) {
         __nv_bfloat162* o = static_cast<__nv_bfloat162*>(out) + ((size_t)sl * Mh + kx) * N;
@@ -765,7 +801,7 @@ __device__ __forceinline__ void dec_group(const float2* X, void* out, const floa
 }
 
 template <int LOG_N, bool S16>
-__global__ void __launch_bounds__(256) k_dec_lines(LinesArgs a) {
+__global__ void __launch_bounds__(256, LOG_N == 10 && !S16 ? 2 : 1) k_dec_lines(LinesArgs a) {
   using P = LinesT<LOG_N>;
   constexpr int T = P::T, R = P::R, N = P::N;
   extern __shared__ float2 smem[];
@@ -798,8 +834,8 @@ struct RecLinesArgs {
 };
 
 template <int LOG_N>
-__global__ void __launch_bounds__(256, LinesT<LOG_N>::R >= 32 ? 1 : 2) k_rec_lines(RecLinesArgs a) {
-  using P = LinesT<LOG_N>;
+__global__ void __launch_bounds__(256, LinesT<LOG_N, true>::R >= 32 ? 1 : 2) k_rec_lines(RecLinesArgs a) {
+  using P = LinesT<LOG_N, true>;
   constexpr int T = P::T, R = P::R, N = P::N, NG = P::NG;
   extern __shared__ float2 smem[];
   float2* red = smem + (size_t)NG * P::C::WORDS;     // [NG][N] partial sums
@@ -840,7 +876,7 @@ __global__ void __launch_bounds__(256, LinesT<LOG_N>::R >= 32 ? 1 : 2) k_rec_lin
     group_sync<T>(1 + g);                   // line read before it is overwritten
     if (s + NG < s_end) fetch(s + NG);
     cp_async_commit();
-    line_fft_any<N, R, -1>(v, line, j, 1 + g, twl, twb);
+    line_fft_any<N, R, -1, true>(v, line, j, 1 + g, twl, twb);
 #pragma unroll
     for (int u = 0; u < R; ++u) {
       const float gv = gok ? __ldg(G + j + u * T) : 0.f;
@@ -873,7 +909,7 @@ __global__ void __launch_bounds__(256, LinesT<LOG_N>::R >= 32 ? 1 : 2) k_rec_lin
     float2 v[R];
 #pragma unroll
     for (int u = 0; u < R; ++u) v[u] = red[j + u * T];
-    line_fft_any<N, R, +1>(v, line, j, 1, twl, twb);
+    line_fft_any<N, R, +1, true>(v, line, j, 1, twl, twb);
 #pragma unroll
     for (int u = 0; u < R; ++u) A[j + u * T] = v[u];
   }
@@ -1115,21 +1151,23 @@ static int sm_count() {
 }
 
 template <int LOG_M>
-static cudaError_t r2c_t(InMode mode, bool th, const RowsTArgs& a, cudaStream_t st) {
+static cudaError_t r2c_t(InMode mode, bool th, bool coeffs, const RowsTArgs& a, cudaStream_t st) {
   using P = RowsT<LOG_M>;
   const int ntiles = a.nsub * (a.N / P::TR);
   if (ntiles == 0) return cudaSuccess;
   cudaError_t e;
-#define SHL_LAUNCH(INM, TH)                                                         \
+#define SHL_LAUNCH(INM, TH, PK)                                                     \
   do {                                                                              \
     const size_t sm = r2c_nst<LOG_M, INM>() * r2c_stage_bytes<LOG_M, INM>() + P::WORK + P::TWB; \
     const int grid = std::min(ntiles, sm_count() * r2c_minb<LOG_M, INM>());         \
-    if ((e = prep(k_rows_r2c_t<LOG_M, INM, TH>, sm))) return e;                     \
-    k_rows_r2c_t<LOG_M, INM, TH><<<grid, P::THREADS, sm, st>>>(a);                   \
+    if ((e = prep(k_rows_r2c_t<LOG_M, INM, TH, PK>, sm))) return e;                 \
+    k_rows_r2c_t<LOG_M, INM, TH, PK><<<grid, P::THREADS, sm, st>>>(a);               \
   } while (0)
-  if (mode == IN_MASKED) SHL_LAUNCH(IN_MASKED, false);
-  else if (mode == IN_BF16) { if (th) SHL_LAUNCH(IN_BF16, true); else SHL_LAUNCH(IN_BF16, false); }
-  else { if (th) SHL_LAUNCH(IN_F32, true); else SHL_LAUNCH(IN_F32, false); }
+  constexpr bool PC = rows_packed<LOG_M>();
+  if (mode == IN_MASKED) SHL_LAUNCH(IN_MASKED, false, false);
+  else if (mode == IN_BF16) { if (th) SHL_LAUNCH(IN_BF16, true, PC); else SHL_LAUNCH(IN_BF16, false, PC); }
+  else if (!coeffs) SHL_LAUNCH(IN_F32, false, false);
+  else { if (th) SHL_LAUNCH(IN_F32, true, PC); else SHL_LAUNCH(IN_F32, false, PC); }
 #undef SHL_LAUNCH
   return cudaGetLastError();
 }
@@ -1194,9 +1232,10 @@ static cudaError_t lines_t(int mode, const LinesArgs& a, const RecLinesArgs& ra,
     else if (a.s16) k_dec_lines<LOG_N, true><<<grid, P::THREADS, sm, st>>>(a);
     else k_dec_lines<LOG_N, false><<<grid, P::THREADS, sm, st>>>(a);
   } else {
-    const size_t sm = P::SMEM_LINES + sizeof(float2) * (size_t)P::NG * P::N + P::TWB;
+    using Q = LinesT<LOG_N, true>;
+    const size_t sm = Q::SMEM_LINES + sizeof(float2) * (size_t)Q::NG * Q::N + Q::TWB;
     if ((e = prep(k_rec_lines<LOG_N>, sm))) return e;
-    k_rec_lines<LOG_N><<<dim3(ra.Mh, grid_y), P::THREADS, sm, st>>>(ra);
+    k_rec_lines<LOG_N><<<dim3(ra.Mh, grid_y), Q::THREADS, sm, st>>>(ra);
   }
   return cudaGetLastError();
 }
@@ -1216,9 +1255,9 @@ static cudaError_t lines_t(int mode, const LinesArgs& a, const RecLinesArgs& ra,
 
 cudaError_t launch_rows_r2c_t(int M, InMode mode, bool thresh, const void* in, const uint8_t* mask,
                               const float* fest, const float* th, float2* out, int N, int nsub,
-                              const float2* tw, cudaStream_t st) {
+                              const float2* tw, cudaStream_t st, bool coeffs) {
   RowsTArgs a{in, mask, fest, th, out, tw, N, nsub};
-#define CALL(X) r2c_t<X>(mode, thresh, a, st)
+#define CALL(X) r2c_t<X>(mode, thresh, coeffs, a, st)
   SHL_SWITCH_LOG(ilog2(M), CALL)
 #undef CALL
 }

@@ -24,6 +24,23 @@ __host__ __device__ constexpr int ilog2(int n) { return n <= 1 ? 0 : 1 + ilog2(n
 
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+// Both components in one packed instruction (add / sub.rn.f32x2: two IEEE additions,
+// one issue slot; the scalar forms may be contracted with a neighbouring multiply).
+// Packed arithmetic issues at half rate, so it saves issue slots, not pipe time.
+__device__ __forceinline__ float2 caddp(float2 a, float2 b) {
+  float2 r;
+  asm("{\n .reg .b64 p, q, s;\n mov.b64 p, {%2, %3};\n mov.b64 q, {%4, %5};\n add.rn.f32x2 s, p, q;\n"
+      " mov.b64 {%0, %1}, s;\n}"
+      : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+__device__ __forceinline__ float2 csubp(float2 a, float2 b) {
+  float2 r;
+  asm("{\n .reg .b64 p, q, s;\n mov.b64 p, {%2, %3};\n mov.b64 q, {%4, %5};\n sub.rn.f32x2 s, p, q;\n"
+      " mov.b64 {%0, %1}, s;\n}"
+      : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
@@ -84,7 +101,10 @@ template <int N> struct BitRev {
 
 // In-register DFT of size R (power of two <= 32), natural order in and out.
 // Radix-2 decimation in frequency followed by a compile-time bit reversal.
-template <int R, int SIGN>
+// PK: packed additions.  They round each addition by itself, where the scalar code
+// is contracted with the multiplies around it, so the passes whose results are
+// stored as bfloat16 (an ulp there is 2^-8) keep the scalar form.
+template <int R, int SIGN, bool PK = false>
 __device__ __forceinline__ void dft_reg(float2* v) {
   if constexpr (R == 1) return;
   else {
@@ -95,8 +115,13 @@ __device__ __forceinline__ void dft_reg(float2* v) {
 #pragma unroll
         for (int q = 0; q < span; ++q) {
           float2 a = v[start + q], b = v[start + q + span];
-          v[start + q] = cadd(a, b);
-          float2 d = csub(a, b);
+          v[start + q] = PK ? caddp(a, b) : cadd(a, b);
+          if (PK && q * (16 / span) == 8) {   // a quarter turn of the difference has no packed form
+            v[start + q + span] = SIGN < 0 ? make_float2(a.y - b.y, b.x - a.x)
+                                           : make_float2(b.y - a.y, a.x - b.x);
+            continue;
+          }
+          float2 d = PK ? csubp(a, b) : csub(a, b);
           // twiddle exp(SIGN 2 pi i q / (2 span)), in 32nds: q * 16 / span
           float2 r;
           switch (q * (16 / span)) {

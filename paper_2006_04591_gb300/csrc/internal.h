@@ -25,7 +25,7 @@ enum InMode : int {
 // [Mh][N] with Mh = M/2 + 1 and the N column-frequency values contiguous.
 cudaError_t launch_rows_r2c_t(int M, InMode mode, bool thresh, const void* in, const uint8_t* mask,
                               const float* fest, const float* th, float2* out, int N, int nsub,
-                              const float2* tw, cudaStream_t st);
+                              const float2* tw, cudaStream_t st, bool coeffs = false);
 // s16: the staged planes are bfloat16 (bfloat16 output only).
 cudaError_t launch_rows_c2r_t(int M, bool bf16, const void* in, void* out, int N, int nsub,
                               const float2* tw, cudaStream_t st, bool s16 = false);

@@ -104,7 +104,7 @@ __device__ __forceinline__ float2 stw(const float2* p) {
 template <int R>
 __device__ __forceinline__ int pad_base(int p) { return p + (p >> ilog2(R)); }
 
-template <int L, int R, int SIGN>
+template <int L, int R, int SIGN, bool PK = false>
 __device__ __forceinline__ void line_fft(float2 (&v)[R], float2* sm, int j, int bar_id,
                                          const float2* __restrict__ stw_sm) {
   using C = LineCfg<L, R>;
@@ -121,7 +121,7 @@ __device__ __forceinline__ void line_fft(float2 (&v)[R], float2* sm, int j, int 
 #pragma unroll
       for (int u = 1; u < R; ++u) v[u] = cmul(v[u], stw<SIGN>(w + (u - 1) * T));
     }
-    dft_reg<R, SIGN>(v);
+    dft_reg<R, SIGN, PK>(v);
     if (st < C::NFULL - 1 || C::LAST > 1) {
       group_sync<T>(bar_id);
       if (st == 0) {
@@ -158,7 +158,7 @@ __device__ __forceinline__ void line_fft(float2 (&v)[R], float2* sm, int j, int 
         w[m] = v[q + m * Q];
         if (m > 0) w[m] = cmul(w[m], stw<SIGN>(wl + (q * (LAST - 1) + (m - 1)) * T));
       }
-      dft_reg<LAST, SIGN>(w);
+      dft_reg<LAST, SIGN, PK>(w);
 #pragma unroll
       for (int m = 0; m < LAST; ++m) v[q + m * Q] = w[m];
     }
@@ -188,13 +188,13 @@ struct LineTwB {
 // exchanges, 4 or 5 shared-memory loads per line instead of 15 or 23
 // (middle stage b^u: products of at most two bases; last stage of 512:
 // w0 times the 16th roots of unity).
-template <int L, int R, int SIGN>
+template <int L, int R, int SIGN, bool PK = false>
 __device__ __forceinline__ void line_fft_b(float2 (&v)[R], float2* sm, int j, int bar_id,
                                            const float2* __restrict__ twb) {
   static_assert(LineTwB<L, R>::OK, "bases exist for 256 and 512 points, radix 16");
   constexpr int T = L / R;
   auto cj = [](float2 a) { return SIGN < 0 ? a : make_float2(a.x, -a.y); };
-  dft_reg<R, SIGN>(v);
+  dft_reg<R, SIGN, PK>(v);
   group_sync<T>(bar_id);
   {
     float2* wp = sm + j * (R + 1);
@@ -215,7 +215,7 @@ __device__ __forceinline__ void line_fft_b(float2 (&v)[R], float2* sm, int j, in
 #pragma unroll
     for (int u = 1; u < R; ++u) v[u] = cmul(v[u], w[u]);
   }
-  dft_reg<R, SIGN>(v);
+  dft_reg<R, SIGN, PK>(v);
   if constexpr (L == 512) {
     group_sync<T>(bar_id);
     {
@@ -241,19 +241,19 @@ __device__ __forceinline__ void line_fft_b(float2 (&v)[R], float2* sm, int j, in
         default: break;
       }
       const float2 x0 = v[q];
-      v[q] = cadd(x0, x1);
-      v[q + R / 2] = csub(x0, x1);
+      v[q] = PK ? caddp(x0, x1) : cadd(x0, x1);
+      v[q + R / 2] = PK ? csubp(x0, x1) : csub(x0, x1);
     }
   }
 }
 
 // line_fft or, where the lane bases exist, line_fft_b.
-template <int L, int R, int SIGN>
+template <int L, int R, int SIGN, bool PK = false>
 __device__ __forceinline__ void line_fft_any(float2 (&v)[R], float2* sm, int j, int bar_id,
                                              const float2* __restrict__ stw_sm,
                                              const float2* __restrict__ twb) {
-  if constexpr (LineTwB<L, R>::OK) line_fft_b<L, R, SIGN>(v, sm, j, bar_id, twb);
-  else line_fft<L, R, SIGN>(v, sm, j, bar_id, stw_sm);
+  if constexpr (LineTwB<L, R>::OK) line_fft_b<L, R, SIGN, PK>(v, sm, j, bar_id, twb);
+  else line_fft<L, R, SIGN, PK>(v, sm, j, bar_id, stw_sm);
 }
 
 // Store v[u] (natural positions j + u T) into the padded line buffer.
