@@ -32,6 +32,7 @@
 //        x[2n] + i x[2n+1] = unnormalised IFFT_L(Z)[n] (= M times the
 //        normalised inverse; 1/(N M) is folded into filter or weight factors).
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdlib>
 
@@ -1204,6 +1205,8 @@ static cudaError_t shrink_t(const RowsShrinkArgs& a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+constexpr int MAX_DEVICES = 16;   // devices whose occupancy is kept
+
 template <int LOG_N>
 static cudaError_t lines_t(int mode, const LinesArgs& a, const RecLinesArgs& ra, int grid_y,
                            cudaStream_t st) {
@@ -1214,18 +1217,21 @@ static cudaError_t lines_t(int mode, const LinesArgs& a, const RecLinesArgs& ra,
     const int work = mode == 1 ? ((a.nlines / a.Mh + DEC_FPG - 1) / DEC_FPG) * a.Mh : a.nlines;
     const size_t sm = P::SMEM_LINES + P::TWB;
     // persistent grid-stride: exactly the CTAs that fit at once, so that no
-    // partial last wave is left
-    int per_sm = 0;
-    if (mode == 0) {
-      if ((e = prep(k_lines_fwd<LOG_N>, sm))) return e;
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lines_fwd<LOG_N>, P::THREADS, sm);
-    } else if (a.s16) {
-      if ((e = prep(k_dec_lines<LOG_N, true>, sm))) return e;
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_dec_lines<LOG_N, true>, P::THREADS, sm);
-    } else {
-      if ((e = prep(k_dec_lines<LOG_N, false>, sm))) return e;
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_dec_lines<LOG_N, false>, P::THREADS, sm);
-    }
+    // partial last wave is left; the count is asked for once per kernel and device
+    const int which = mode == 0 ? 0 : a.s16 ? 1 : 2;
+    static std::atomic<int> cached[3][MAX_DEVICES];
+    int dev = 0;
+    if ((e = cudaGetDevice(&dev))) return e;
+    int per_sm = dev < MAX_DEVICES ? cached[which][dev].load(std::memory_order_relaxed) : 0;
+    auto ask = [&](auto kernel) -> cudaError_t {
+      cudaError_t r = prep(kernel, sm);
+      if (r || per_sm) return r;
+      r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, P::THREADS, sm);
+      if (!r && dev < MAX_DEVICES) cached[which][dev].store(per_sm, std::memory_order_relaxed);
+      return r;
+    };
+    e = which == 0 ? ask(k_lines_fwd<LOG_N>) : which == 1 ? ask(k_dec_lines<LOG_N, true>)
+                                                          : ask(k_dec_lines<LOG_N, false>);
     if (e) return e;
     const int grid = std::max(1, std::min((work + P::NG - 1) / P::NG, std::max(per_sm, 1) * sm_count()));
     if (mode == 0) k_lines_fwd<LOG_N><<<grid, P::THREADS, sm, st>>>(a);

@@ -1013,9 +1013,11 @@ cudaError_t launch_tc(const ConvTcArgs& a, cudaStream_t st) {
   // TMEM columns.  No CTA
   // waits on another, so the count only sizes the grid.
   int per_sm = (int)((228u * 1024u) / (P::SMEM + 1024u + 256u));
-  cudaFuncAttributes fa{};
-  if (cudaFuncGetAttributes(&fa, k) == cudaSuccess && fa.numRegs > 0)
-    per_sm = std::min(per_sm, 65536 / (fa.numRegs * CONV_THREADS));
+  static const int regs = [k] {                 // a property of the kernel, asked for once
+    cudaFuncAttributes fa{};
+    return cudaFuncGetAttributes(&fa, k) == cudaSuccess ? fa.numRegs : 0;
+  }();
+  if (regs > 0) per_sm = std::min(per_sm, 65536 / (regs * CONV_THREADS));
   per_sm = std::max(1, std::min({per_sm, 8, (int)(512 / P::NCOLS)}));
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);

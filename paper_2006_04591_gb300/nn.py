@@ -20,6 +20,7 @@ tape; every arithmetic step calls the library.
 from __future__ import annotations
 
 import ctypes
+import functools
 import math
 
 import numpy as np
@@ -87,11 +88,11 @@ def _chk(name, st):
 
 
 def _p(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _st(t):
-    return ctypes.c_void_p(torch.cuda.current_stream(t.device).cuda_stream)
+    return S.current_stream_ptr(t.device)
 
 
 def _ws(n, like):
@@ -110,6 +111,7 @@ def _chk_tc(name, st):
         raise S.ShearletError(name, st, lib().shl_nn_tc_last_error().decode())
 
 
+@functools.lru_cache(maxsize=256)
 def shl_nn_conv3x3_tc_supported(Ci, Co, H, W):
     return bool(lib().shl_nn_conv3x3_tc_supported(Ci, Co, H, W))
 
@@ -126,6 +128,7 @@ def shl_nn_conv3x3_backward_data_tc(gout, w, gin):
         _p(gout), _p(w), _p(gin), B, Ci, w.shape[0], H, W, _st(gin)))
 
 
+@functools.lru_cache(maxsize=256)
 def shl_nn_conv3x3_wgrad_tc_supported(Ci, Co, H, W):
     return bool(lib().shl_nn_conv3x3_wgrad_tc_supported(Ci, Co, H, W))
 

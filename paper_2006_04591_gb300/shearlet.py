@@ -117,16 +117,27 @@ def _check(fn, status):
 
 
 def _ptr(t):
-    if t is None:
-        return None
-    return ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()   # an int: the declared argtypes convert it
+
+
+def current_stream_ptr(device):
+    """The cudaStream_t (an int) of torch's current stream on ``device`` (a torch
+    device or an index), without the Stream object that
+    torch.cuda.current_stream() builds around it on every call."""
+    import torch
+    if isinstance(device, int):
+        index = device
+    elif device.type == "cuda":
+        index = device.index
+    else:
+        raise ValueError("expected a CUDA device, got %s" % device)
+    if index is None:
+        index = torch.cuda.current_device()
+    return torch._C._cuda_getCurrentRawStream(index)
 
 
 def _stream(stream, device):
-    import torch
-    if stream is None:
-        stream = torch.cuda.current_stream(device)
-    return ctypes.c_void_p(stream.cuda_stream)
+    return current_stream_ptr(device) if stream is None else stream.cuda_stream
 
 
 def _dtype_code(dt):
@@ -373,6 +384,7 @@ class Bank:
         self.idx, self.rms = info["idx"], info["rms"]
         self.general = bool(shl_bank_path(handle))
         self._rms_dev = None
+        self._ws_bytes = {}
 
     @classmethod
     def create(cls, rows, cols, n_scales, shear_levels=None, full=False, device=0, on_gpu=False):
@@ -475,7 +487,11 @@ class Bank:
 
     def workspace(self, op, batch):
         import torch
-        n = shl_workspace_size(self.handle, op, batch)
+        n = self._ws_bytes.get((op, batch))
+        if n is None:
+            n = shl_workspace_size(self.handle, op, batch)
+            if len(self._ws_bytes) < 64:
+                self._ws_bytes[op, batch] = n
         return torch.empty(max(n, 16), dtype=torch.uint8, device="cuda:%d" % self.device)
 
     def _check_images(self, x):
