@@ -180,9 +180,9 @@ __global__ void __launch_bounds__(FWD_BINS) k_ray_forward(const float* __restric
 // hat weight 1 - |u - k|: exactly the forward's 1 - w1 or w1, since u - k and
 // the difference from 1 on the far side are exact in float32.  The bins start at
 // the one below the fractional bin of u = k - 1; ADJ_MARGIN covers the rounding
-// of that bin (below 0.01 over the accepted sizes).  What bounds it: issue, about
-// 50 instructions per pixel and angle for four images, whose position, weights
-// and address they share.  Measured as above: 1770 us with one thread
+// of that bin (below 0.01 over the accepted sizes).  What bounds it: the
+// bins' reads through L1, shared by nothing but the four images' position, weights
+// and address.  Measured as above: 1770 us with one thread
 // per pixel and image (a floor and a compare per candidate bin), 527 us so; 32
 // images of 128 x 128 at 30 angles: 96 and 33 us (forward 107 and 45 us).
 constexpr float ADJ_MARGIN = 0.05f;
@@ -244,6 +244,99 @@ __global__ void __launch_bounds__(256) k_ray_adjoint(const float* __restrict__ s
         img[((size_t)(b0 + b) * n + i0 + 8 * x) * n + j] = acc[x][b];
 }
 
+// The same with the bins that a tile of 32 x 32 pixels can receive staged in shared
+// memory, images interleaved: one NB-wide read per bin in place of NB gathers
+// through L1.  Chunks of `ac` angles, W bins each; lo_of the first staged bin.
+constexpr int ADJ_TILE_PIX = 4;    // pixels per thread, 8 rows apart
+constexpr int ADJ_CHUNK = 16;      // most angles staged at a time
+constexpr size_t ADJ_SMEM = 48 * 1024;
+constexpr double ADJ_TILE_BINS = 160;   // widest staging of one angle
+
+template <int NB>
+__global__ void __launch_bounds__(256) k_ray_adjoint_tile(const float* __restrict__ sino,
+                                                          float* __restrict__ img,
+                                                          const AngleParam* __restrict__ prm, int n,
+                                                          int A, int D, int B, int W, int ac) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  Vec<NB>* S = reinterpret_cast<Vec<NB>*>(smem);     // [ac][W]
+  __shared__ int s_lo[ADJ_CHUNK];
+  const int tid = threadIdx.x;
+  const int j0 = blockIdx.x * 32, r0 = blockIdx.y * (8 * ADJ_TILE_PIX), b0 = blockIdx.z * NB;
+  const int j = j0 + (tid & 31), i0 = r0 + (tid >> 5);
+  const float* p[NB];
+#pragma unroll
+  for (int b = 0; b < NB; ++b) p[b] = sino + (size_t)min(b0 + b, B - 1) * A * D;
+  float acc[ADJ_TILE_PIX][NB];
+#pragma unroll
+  for (int x = 0; x < ADJ_TILE_PIX; ++x)
+#pragma unroll
+    for (int b = 0; b < NB; ++b) acc[x][b] = 0.f;
+  for (int a0 = 0; a0 < A; a0 += ac) {
+    const int na = min(ac, A - a0);
+    __syncthreads();                                 // the earlier bins have been read
+    if (tid < na) {
+      // smallest fractional bin over the tile's corners (it is affine in t and k)
+      const AngleParam q = load_angle(prm + a0 + tid);
+      const int t0 = q.by_rows ? r0 : j0, k0 = q.by_rows ? j0 : r0;
+      float lo = 1e30f;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const float t = (float)(t0 + (c & 1) * 31), k = (float)(k0 + (c >> 1) * 31);
+        lo = fminf(lo, (k - fmaf(q.B, t, q.C)) * q.inv_a);
+      }
+      s_lo[tid] = (int)floorf(fminf(fmaxf(lo - fabsf(q.inv_a) - ADJ_MARGIN, -1e6f), 1e6f)) - 1;
+    }
+    __syncthreads();
+    for (int idx = tid; idx < na * W; idx += 256) {
+      const int a = idx / W, d = s_lo[a] + idx - a * W;
+      Vec<NB> v;
+#pragma unroll
+      for (int b = 0; b < NB; ++b)
+        v.v[b] = d >= 0 && d < D ? __ldg(p[b] + (size_t)(a0 + a) * D + d) : 0.f;
+      S[idx] = v;
+    }
+    __syncthreads();
+    for (int a = 0; a < na; ++a) {
+      const AngleParam q = load_angle(prm + a0 + a);
+      const float first = fabsf(q.inv_a) + (ADJ_MARGIN + 0.5f);
+      const int lo0 = s_lo[a];
+      const Vec<NB>* s = S + a * W;
+#pragma unroll
+      for (int x = 0; x < ADJ_TILE_PIX; ++x) {
+        const int i = i0 + 8 * x;
+        const float t = (float)(q.by_rows ? i : j), k = (float)(q.by_rows ? j : i);
+        const float base = fmaf(q.B, t, q.C);
+        int lo;
+        const float flo = round_near(fminf(fmaxf((k - base) * q.inv_a - first, -1e6f), 1e6f), &lo);
+        const Vec<NB>* r = s + min(max(lo - lo0, 0), W - q.bins);
+        float sa[NB];
+#pragma unroll
+        for (int b = 0; b < NB; ++b) sa[b] = 0.f;
+        auto bin = [&](int m) {
+          const float w = __saturatef(1.f - fabsf(fmaf(q.A, flo + (float)m, base) - k));
+          const Vec<NB> v = r[m];
+          if (w > 0.f) {               // a bin outside the hat does not enter the sum
+#pragma unroll
+            for (int b = 0; b < NB; ++b) sa[b] = fmaf(w, v.v[b], sa[b]);
+          }
+        };
+        bin(0);
+        bin(1);
+        if (q.bins > 2) bin(2);
+        for (int m = 3; m < q.bins; ++m) bin(m);
+#pragma unroll
+        for (int b = 0; b < NB; ++b) acc[x][b] = fmaf(sa[b], q.w, acc[x][b]);
+      }
+    }
+  }
+#pragma unroll
+  for (int x = 0; x < ADJ_TILE_PIX; ++x)
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+      if (j < n && i0 + 8 * x < n && b0 + b < B)
+        img[((size_t)(b0 + b) * n + i0 + 8 * x) * n + j] = acc[x][b];
+}
+
 bool aligned4(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 3u) == 0; }
 
 }  // namespace
@@ -255,6 +348,8 @@ struct shl_ray {
   int ngrp = 0;
   double a_max = 0, b_max = 0;      // largest |A| and |B| over the angles
   double pair_max = 0;              // largest |u - u'| between the angles of a group
+  double inv_max = 0, tile_max = 0; // largest 1/|A| and (1 + |B|)/|A|
+  int sms = 1;
 };
 
 namespace {
@@ -262,10 +357,7 @@ namespace {
 // Images per CTA: the position and the weights of a sample are shared by the
 // images, so as many as there are (up to four) unless the launch would then
 // leave SMs without two CTAs.
-int images_per_cta(long long ctas_per_image, int batch) {
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+int images_per_cta(int sms, long long ctas_per_image, int batch) {
   for (int nb = 4; nb > 1; nb /= 2)
     if (batch >= nb && ctas_per_image * ((batch + nb - 1) / nb) >= 2LL * sms) return nb;
   return 1;
@@ -295,6 +387,18 @@ cudaError_t forward_nb(const shl_ray* op, const float* img, int batch, float* si
 
 template <int NB>
 cudaError_t adjoint_nb(const shl_ray* op, const float* sino, int batch, float* img, cudaStream_t st) {
+  // bins a tile can receive from one angle (31 pixels along each axis, the hat's
+  // width, the margins and the rounding of the first bin)
+  const double reach = 31.0 * op->tile_max + 2.0 * op->inv_max + 6.0;
+  const long long tiles = (op->n + 31LL) / 32 * ((op->n + 31) / 32) * ((batch + NB - 1) / NB);
+  if (reach <= ADJ_TILE_BINS && tiles >= 2LL * op->sms) {
+    const int W = (int)reach + 1;
+    const int ac = (int)std::min<size_t>(ADJ_CHUNK, ADJ_SMEM / (W * sizeof(Vec<NB>)));
+    const dim3 grid((op->n + 31) / 32, (op->n + 31) / 32, (batch + NB - 1) / NB);
+    k_ray_adjoint_tile<NB><<<grid, 256, (size_t)ac * W * sizeof(Vec<NB>), st>>>(
+        sino, img, op->dPrm, op->n, op->A, op->D, batch, W, ac);
+    return cudaGetLastError();
+  }
   const dim3 grid((op->n + 31) / 32, (op->n + 8 * ADJ_PIX - 1) / (8 * ADJ_PIX), (batch + NB - 1) / NB);
   k_ray_adjoint<NB><<<grid, 256, 0, st>>>(sino, img, op->dPrm, op->n, op->A, op->D, batch);
   return cudaGetLastError();
@@ -334,8 +438,10 @@ shl_status shl_ray_create(int n, int n_angles, int n_det, int device, shl_ray** 
   // the corners bound the difference)
   constexpr double PAIR_PIXELS = 64.0;
   std::vector<AngleGroup> grp;
-  double a_max = 0, b_max = 0, pair_max = 0;
+  double a_max = 0, b_max = 0, pair_max = 0, inv_max = 0, tile_max = 0;
   for (const AngleParam& q : prm) {
+    inv_max = std::max(inv_max, (double)std::fabs(q.inv_a));
+    tile_max = std::max(tile_max, (1.0 + std::fabs(q.B)) * std::fabs(q.inv_a));
     a_max = std::max(a_max, (double)std::fabs(q.A));
     b_max = std::max(b_max, (double)std::fabs(q.B));
   }
@@ -362,6 +468,8 @@ shl_status shl_ray_create(int n, int n_angles, int n_det, int device, shl_ray** 
   op->device = device; op->n = n; op->A = n_angles; op->D = n_det;
   op->ngrp = (int)grp.size();
   op->a_max = a_max; op->b_max = b_max; op->pair_max = pair_max;
+  op->inv_max = inv_max; op->tile_max = tile_max;
+  cudaDeviceGetAttribute(&op->sms, cudaDevAttrMultiProcessorCount, device);
   cudaError_t e = cudaMalloc(&op->dPrm, sizeof(AngleParam) * n_angles);
   if (!e) e = cudaMalloc(&op->dGrp, sizeof(AngleGroup) * grp.size());
   if (!e) e = cudaMemcpy(op->dPrm, prm.data(), sizeof(AngleParam) * n_angles, cudaMemcpyHostToDevice);
@@ -415,7 +523,7 @@ shl_status shl_ray_forward(const shl_ray* op, const float* img, int batch, float
     const float* x = img + (size_t)b0 * op->n * op->n;
     float* y = sino + (size_t)b0 * op->A * op->D;
     const cudaStream_t st = static_cast<cudaStream_t>(stream);
-    switch (images_per_cta((op->D + FWD_BINS - 1LL) / FWD_BINS * op->ngrp, nb)) {
+    switch (images_per_cta(op->sms, (op->D + FWD_BINS - 1LL) / FWD_BINS * op->ngrp, nb)) {
       case 4: e = forward_nb<4>(op, x, nb, y, st); break;
       case 2: e = forward_nb<2>(op, x, nb, y, st); break;
       default: e = forward_nb<1>(op, x, nb, y, st); break;
@@ -441,7 +549,7 @@ shl_status shl_ray_adjoint(const shl_ray* op, const float* sino, int batch, floa
     const float* y = sino + (size_t)b0 * op->A * op->D;
     float* x = img + (size_t)b0 * op->n * op->n;
     const cudaStream_t st = static_cast<cudaStream_t>(stream);
-    switch (images_per_cta((op->n + 31LL) / 32 * ((op->n + 8 * ADJ_PIX - 1) / (8 * ADJ_PIX)), nb)) {
+    switch (images_per_cta(op->sms, (op->n + 31LL) / 32 * ((op->n + 8 * ADJ_PIX - 1) / (8 * ADJ_PIX)), nb)) {
       case 4: e = adjoint_nb<4>(op, y, nb, x, st); break;
       case 2: e = adjoint_nb<2>(op, y, nb, x, st); break;
       default: e = adjoint_nb<1>(op, y, nb, x, st); break;
