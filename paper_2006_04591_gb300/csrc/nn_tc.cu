@@ -402,8 +402,11 @@ struct WgradTcT {
   static constexpr int THREADS = 512;                       // 16 warps stage, 4 read TMEM
   static constexpr int PG = TC_M / 8;                       // pixel groups per unit row
   static constexpr int SLOTS = 4;                           // input-row ring
-  static constexpr size_t ABYTES = (size_t)PG * 128 * 16;   // one input row: [pg][r][8]
-  static constexpr size_t BBYTES = (size_t)PG * NP * 16;    // one gout row: [pg][o][8]
+  // A pixel group's rows are followed by 16 bytes, so that the 16 groups of one
+  // channel, which consecutive threads store, meet no bank twice.
+  static constexpr uint32_t ASTR = 128 * 16 + 16, BSTR = NP * 16 + 16;
+  static constexpr size_t ABYTES = (size_t)PG * ASTR;       // one input row: [pg][r][8]
+  static constexpr size_t BBYTES = (size_t)PG * BSTR;       // one gout row: [pg][o][8]
   static constexpr size_t SMEM = SLOTS * ABYTES + 2 * BBYTES;
   static constexpr uint32_t NCOLS =
       3 * NP <= 64 ? 64 : (3 * NP <= 128 ? 128 : (3 * NP <= 256 ? 256 : 512));
@@ -414,8 +417,11 @@ struct WgradTcT {
 // Staging of the weight-gradient operands in two halves, so that the global
 // loads of the next rows are in flight while the MMAs of the current row
 // run: *_load fills registers, *_store converts them to bfloat16 and writes
-// shared memory.  Item idx -> (pixel group pg = idx / C, channel idx % C):
-// consecutive threads write consecutive 16-byte rows (no bank conflicts).
+// shared memory.  Item idx -> (channel idx / PG, pixel group idx % PG): consecutive
+// threads read consecutive 32 bytes of one channel's row.  (With the channel
+// running first every load of a warp touched 32 lines of 32 channels, which bound
+// the kernel: 32 x 256^2, 33 -> 32 channels, 267 -> 200 us; with the
+// addresses formed per unit and 512 threads, 353 us before all three.)
 template <int NP>
 struct WgradRegs {
   float e[WgradTcT<NP>::IITEMS][10];     // input: pixels x0+8pg-1 .. x0+8pg+8
@@ -436,17 +442,17 @@ __device__ __forceinline__ void wgrad_src(const WgradTcArgs& a, WgradSrc<NP>& s,
   using P = WgradTcT<NP>;
 #pragma unroll
   for (int k = 0; k < P::IITEMS; ++k) {
-    const int idx = tid + k * P::THREADS, pg = idx / a.Cin, i = idx - pg * a.Cin;
+    const int idx = tid + k * P::THREADS, i = idx / P::PG, pg = idx % P::PG;
     s.ix[k] = x0 + 8 * pg;
-    s.di[k] = (pg * 128 + i) * 16;
-    s.in[k] = pg < P::PG ? a.in + ((size_t)b * a.Ctot + i) * a.H * a.W + s.ix[k] : nullptr;
+    s.di[k] = pg * P::ASTR + i * 16;
+    s.in[k] = i < a.Cin ? a.in + ((size_t)b * a.Ctot + i) * a.H * a.W + s.ix[k] : nullptr;
   }
 #pragma unroll
   for (int k = 0; k < P::BITEMS; ++k) {
-    const int idx = tid + k * P::THREADS, pg = idx / a.Cout, o = idx - pg * a.Cout;
+    const int idx = tid + k * P::THREADS, o = idx / P::PG, pg = idx % P::PG;
     s.gx[k] = x0 + 8 * pg;
-    s.dg[k] = (pg * NP + o) * 16;
-    s.g[k] = pg < P::PG ? a.gout + ((size_t)b * a.Cout + o) * a.H * a.W + s.gx[k] : nullptr;
+    s.dg[k] = pg * P::BSTR + o * 16;
+    s.g[k] = o < a.Cout ? a.gout + ((size_t)b * a.Cout + o) * a.H * a.W + s.gx[k] : nullptr;
   }
 }
 
@@ -526,7 +532,7 @@ __device__ __forceinline__ void wgrad_load_gout(const WgradTcArgs& a, const Wgra
 }
 
 // -> B[o][p] = gout[o][y][x0 + p]; bsum[k] gathers this thread's float32
-// bias partial (item k always has channel (tid + k THREADS) mod Cout)
+// bias partial (item k always has the same channel)
 template <int NP>
 __device__ __forceinline__ void wgrad_store_gout(const WgradSrc<NP>& s, const WgradRegs<NP>& R,
                                                  uint8_t* dst, float (&bsum)[WgradTcT<NP>::BITEMS]) {
@@ -624,8 +630,8 @@ __global__ void __launch_bounds__(WgradTcT<NP>::THREADS, 1) k_wgrad_tc(const Wgr
           const uint32_t brow = bbase + (uint32_t)((y & 1) * P::BBYTES);
 #pragma unroll
           for (int s = 0; s < P::PG / 2; ++s) {
-            const uint64_t ad = mdesc(arow + (uint32_t)(2 * s * 128 * 16), 128 * 16, 128);
-            const uint64_t bd = mdesc(brow + (uint32_t)(2 * s * NP * 16), NP * 16, 128);
+            const uint64_t ad = mdesc(arow + 2 * s * P::ASTR, P::ASTR, 128);
+            const uint64_t bd = mdesc(brow + 2 * s * P::BSTR, P::BSTR, 128);
             const uint32_t acc = (first && s == 0) ? 0u : 1u;
             asm volatile(
                 "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
@@ -673,9 +679,9 @@ __global__ void __launch_bounds__(WgradTcT<NP>::THREADS, 1) k_wgrad_tc(const Wgr
   }
   __syncthreads();
   const size_t stride = (size_t)a.Cout * a.Ctot * 9 + a.Cout;
-  if (c0 == 0 && tid < a.Cout) {   // items of channel o: idx = pg * Cout + o
+  if (c0 == 0 && tid < a.Cout) {   // items of channel o: idx = o * PG + pg
     float s = 0.f;
-    for (int pg = 0; pg < P::PG; ++pg) s += bred[pg * a.Cout + tid];
+    for (int pg = 0; pg < P::PG; ++pg) s += bred[tid * P::PG + pg];
     a.part[(size_t)blockIdx.x * stride + (size_t)a.Cout * a.Ctot * 9 + tid] = s;
   }
   // epilogue (warps 0-3): lane r = dx * Cin + i, columns dy * NP + o
