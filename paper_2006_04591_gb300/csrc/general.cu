@@ -1,6 +1,6 @@
 // general.cu - transform kernels for any image size and for complex
-// Hermitian filter spectra (lengths A B with A, B <= 32, and Bluestein lengths up to
-// 512: general_pairs.cuh): the decomposition, reconstruction and adjoint of
+// Hermitian filter spectra (lengths A B with A, B <= 32, and lengths up to 512 with a
+// prime factor above 19: general_pairs.cuh): the decomposition, reconstruction and adjoint of
 // Sec. 3.4 on row-major half-spectrum planes [N][M/2+1] in natural DFT order
 // (real images and Hermitian filters give Hermitian spectra, so columns
 // 0..M/2 determine the rest).
@@ -45,6 +45,7 @@
 #include <cmath>
 #include <complex>
 
+#include "dft_small.cuh"
 #include "general.h"
 #include "general_pairs_list.h"
 
@@ -666,12 +667,19 @@ int pair_part(int A, int B, bool bl) {
 }
 
 // The pair for lines of length L: L itself where it is one of the products; else,
-// where L has a prime factor above BLUESTEIN_PRIME (the one-output-per-thread stages
-// of this file), the shortest Bluestein length.  A = 0 otherwise.  Lengths with
-// factors up to 7 only and no pair keep the direct stages: at 350 rows these take
-// 9.1 (decomposition) and 17.9 (reconstruction) ns per thousand elements, Bluestein
-// at 222 rows 11.9 and 14.3.
-constexpr int BLUESTEIN_PRIME = 7;
+// where L has a prime factor above BLUESTEIN_PRIME, the Bluestein length, the power of
+// two >= 2L - 1 (or the shortest that there is).  A = 0 otherwise.
+//
+// Where the line lies is a matter of rounding, as Bluestein's two transforms were the
+// faster at every length measured (16 x L^2, from 1.1 times at 11 to 2.8 at 61).  RMS
+// error against float64 at all 241 lengths up to 512 with a largest prime factor of 11
+// to 61, Bluestein's over the direct stages', decomposition: on average 1.13 at a factor
+// of 11 (up to 1.32), 1.06 at 13, 1.01 at 17, 0.97 at 19 (up to 1.09), 0.87 at 23 down to
+// 0.63 at 61 and nowhere above 0.98 from 23 on; so lengths with factors up to 19 keep
+// the direct stages.  Convolution lengths between the powers of two ran up to 1.6 times
+// as fast, with up to 1.17 times the error of the power of two: the share L / P of a
+// convolution's rounding is kept.
+constexpr int BLUESTEIN_PRIME = 19;
 PairPlan find_pair(int L) {
   PairPlan p{};
   p.L = L;
@@ -742,29 +750,83 @@ int rec_groups(long long ctas, long long per_sm, int subbands) {
 
 }  // namespace
 
-// Forward DFT in float64 of any length: radix 2 where it is a power of two, else
-// through a power-of-two convolution (Bluestein).
-static void dft_any(std::vector<cd>& x) {
-  const long long n = (long long)x.size();
-  if ((n & (n - 1)) == 0) {
-    fft_pow2(x, -1);
-    return;
+// The two-stage transforms as the kernels run them (dft_small.cuh, general_pairs.cuh),
+// in float64 but with the roots that the kernels have rounded to float32.
+static cd rounded_root(long long k, long long n) {
+  return cd((float)cos_turn(k, n), -(float)sin_turn(k, n));
+}
+static void dft_rounded(cd* v, int r) {                      // r = 2, 4, 8, 16, 32
+  if (r == 1) return;
+  cd out[32], c[32];
+  if (r <= 8) {                                            // dft_reg
+    const int h = r / 2;
+    cd *e = c, *o = c + h;
+    for (int q = 0; q < h; ++q) {
+      e[q] = v[q] + v[q + h];
+      o[q] = (v[q] - v[q + h]) * rounded_root(q, r);
+    }
+    dft_rounded(e, h);
+    dft_rounded(o, h);
+    for (int q = 0; q < r; ++q) out[q] = q % 2 ? o[q / 2] : e[q / 2];
+  } else {                                                 // dft_split<r, 4>
+    const int b = r / 4;
+    cd t[4][8];
+    for (int n2 = 0; n2 < b; ++n2) {
+      for (int n1 = 0; n1 < 4; ++n1) c[n1] = v[b * n1 + n2];
+      dft_rounded(c, 4);
+      for (int k1 = 0; k1 < 4; ++k1) t[k1][n2] = c[k1] * rounded_root(k1 * n2, r);
+    }
+    for (int k1 = 0; k1 < 4; ++k1) {
+      dft_rounded(t[k1], b);
+      for (int k2 = 0; k2 < b; ++k2) out[k1 + 4 * k2] = t[k1][k2];
+    }
   }
-  size_t m = 1;
-  while ((long long)m < 2 * n - 1) m <<= 1;
-  std::vector<cd> c(n), a(m, cd(0, 0)), h(m, cd(0, 0));
-  for (long long k = 0; k < n; ++k) {
-    const double t = -PI * (double)((k * k) % (2 * n)) / (double)n;
-    c[k] = cd(std::cos(t), std::sin(t));
-    a[k] = x[k] * c[k];
-    h[k] = std::conj(c[k]);
-    if (k) h[m - k] = std::conj(c[k]);
+  std::copy(out, out + r, v);
+}
+static std::vector<cd> pair_rounded(const std::vector<cd>& x, int A, int B) {
+  cd u[32][32];
+  for (int j = 0; j < B; ++j) {
+    cd v[32];
+    for (int m = 0; m < A; ++m) v[m] = x[j + m * B];
+    dft_rounded(v, A);
+    for (int k = 0; k < A; ++k) u[k][j] = v[k] * rounded_root((long long)j * k, A * B);
   }
-  fft_pow2(a, -1);
-  fft_pow2(h, -1);
-  for (size_t k = 0; k < m; ++k) a[k] *= h[k];
-  fft_pow2(a, +1);
-  for (long long k = 0; k < n; ++k) x[k] = c[k] * a[k] / (double)m;
+  std::vector<cd> y(x.size());
+  for (int k = 0; k < A; ++k) {
+    dft_rounded(u[k], B);
+    for (int q = 0; q < B; ++q) y[k + q * A] = u[k][q];
+  }
+  return y;
+}
+
+// Mean gain, less 1, of a pair's Bluestein transform with all its tables rounded: over
+// frequency 0 (a constant line's X[0], an impulse at 0), where images have most of
+// their energy, and over impulses along the line, in equal parts.
+static double pair_gain(int L, int A, int B, const std::vector<cd>& chirp, const std::vector<cd>& kern) {
+  auto rnd = [](cd z) { return cd((float)z.real(), (float)z.imag()); };
+  auto run = [&](int lo, int hi) {                         // ones at lo .. hi - 1
+    std::vector<cd> x(kern.size(), cd(0, 0));
+    for (int e = lo; e < hi; ++e) x[e] = rnd(chirp[e]);
+    x = pair_rounded(x, A, B);
+    for (size_t k = 0; k < x.size(); ++k) x[k] = std::conj(x[k] * rnd(kern[k]));
+    x = pair_rounded(x, B, A);
+    for (int k = 0; k < L; ++k) x[k] = rnd(chirp[k]) * std::conj(x[k]);
+    return x;
+  };
+  auto impulse = [&](int n) {
+    const std::vector<cd> x = run(n, n + 1);
+    double g = 0.0;
+    for (int k = 0; k < L; ++k) {
+      const double t = 2.0 * PI * (double)((long long)n * k % L) / L;
+      g += (x[k] * cd(std::cos(t), std::sin(t))).real() / L;
+    }
+    return g;
+  };
+  const double dc = 0.5 * (run(0, L)[0].real() / L + impulse(0));
+  constexpr int N = 16;
+  double along = 0.0;
+  for (int i = 0; i < N; ++i) along += impulse((2 * i + 1) * L / (2 * N)) / N;
+  return 0.5 * (dc + along) - 1.0;
 }
 
 LineTables make_line_tables(int L) {
@@ -807,11 +869,20 @@ LineTables make_line_tables(int L) {
       h[m] = std::conj(c[m]);
       if (m) h[P - m] = std::conj(c[m]);
     }
-    dft_any(h);
+    fft_pow2(h, -1);
+    for (cd& v : h) v /= (double)P;
+    // The roots of a pair's transforms, rounded to float32, scale every line the same
+    // way, by -2e-8 to -8e-8 a transform: -2.5e-7 in the smooth parts of an image of
+    // 440^2 after two row and two column passes, as much as all other rounding
+    // together.  The kernel takes it back.
+    if (q.A) {
+      const double g = 1.0 + pair_gain(L, q.A, q.B, c, h);
+      for (cd& v : h) v /= g;
+    }
     t.off_chirp = t.data.size();
     for (int n = 0; n < L; ++n) t.data.push_back(to_f2(c[n]));
     t.off_kern = t.data.size();
-    for (int k = 0; k < P; ++k) t.data.push_back(to_f2(h[k] / (double)P));
+    for (int k = 0; k < P; ++k) t.data.push_back(to_f2(h[k]));
   }
   return t;
 }

@@ -11,8 +11,8 @@
 // factors <= 61), or with Bluestein's chirp-z algorithm (a larger prime
 // factor: the length-L DFT becomes a circular convolution of length P = the
 // power of two >= 2L - 1).  Lengths that are products of two small radices, and
-// Bluestein lengths up to 512, run on the two-stage register kernels of
-// general_pairs.cuh.
+// lengths up to 512 with a prime factor above 19 (by Bluestein), run on the two-stage
+// register kernels of general_pairs.cuh.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -35,7 +35,8 @@ struct PairPlan {
   const float2* ab;          // [(m - 1) A + k] = exp(-2 pi i m k / P), m < B, k < A
   const float2* ba;          // [(m - 1) B + k], m < A, k < B
   const float2* chirp;       // [L] exp(-i pi n^2 / L) (Bluestein)
-  const float2* kern;        // [P] DFT_P(h) / P, h[m] = conj chirp[|m|]
+  const float2* kern;        // [P] DFT_P(h) / P over the transform's mean gain (pair_gain),
+                             // h[m] = conj chirp[|m|]
 };
 
 // Forward DFT of length L, X[k] = sum_n x[n] exp(-2 pi i n k / L); the

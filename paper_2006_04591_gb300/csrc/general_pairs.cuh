@@ -13,11 +13,13 @@
 // (K = 49, float32, decomposition and reconstruction): 16 x 480 x 640 5375 -> 1806 us
 // (column pass of the reconstruction 1864 -> 395, of the decomposition 1124 -> 417,
 // row passes 1166 -> 452 and 1127 -> 517), 16 x 500^2 4345 -> 1503 us, 4 x 509^2
-// (Bluestein, P = 1024) 3992 -> 1262 us, 16 x 222 x 301 (Bluestein) 4134 -> 1314 us.
+// (Bluestein, P = 1024) 3992 -> 1262 us; with K = 17, 16 x 222 x 301 (Bluestein,
+// P = 512 and 1024) 1575 -> 599 us.
 // At 480 x 640 the passes now run at 35-55 % of the DRAM rate of the planes and
 // coefficients that they move; what is left is latency at 18 to 24 warps per SM.
 //
-// Other lengths up to 512 go through Bluestein's chirp-z identity
+// Lengths up to 512 with a prime factor above 19 (find_pair) go through Bluestein's
+// chirp-z identity
 // n k = (n^2 + k^2 - (k - n)^2)/2 with a pair P >= 2L - 1:
 //   X[k] = c[k] sum_n (x[n] c[n]) conj(c[k - n]),  c[n] = exp(-i pi n^2 / L),
 // a circular convolution of length P evaluated with two length-P FFTs against
