@@ -88,6 +88,9 @@ def _chk(name, st):
 
 
 def _p(t):
+    """Address of a tensor that a local name (or the caller) keeps alive until the
+    launch: the address alone does not, and the allocator may hand the memory of a
+    temporary to the next one."""
     return None if t is None else t.data_ptr()
 
 
@@ -327,10 +330,11 @@ class _PReLU(torch.autograd.Function):
     @staticmethod
     def backward(ctx, gy):
         x, a = ctx.saved_tensors
+        gy = gy.contiguous()
         gx = torch.empty_like(x)
         ga = torch.empty(1, dtype=torch.float32, device=x.device)
         ws = _ws(lib().shl_nn_reduce_workspace_floats(x.numel()), x)
-        _chk("prelu_backward", lib().shl_nn_prelu_backward(_p(x), _p(a), _p(gy.contiguous()), _p(gx),
+        _chk("prelu_backward", lib().shl_nn_prelu_backward(_p(x), _p(a), _p(gy), _p(gx),
                                                             _p(ga), x.numel(), _p(ws), _st(x)))
         return gx, ga.reshape(a.shape)
 
@@ -339,16 +343,18 @@ class _GAP(torch.autograd.Function):
     @staticmethod
     def forward(ctx, x):
         B, C, H, W = x.shape
+        x = x.contiguous()
         y = torch.empty((B, C), dtype=torch.float32, device=x.device)
-        _chk("gap_forward", lib().shl_nn_gap_forward(_p(x.contiguous()), _p(y), B, C, H * W, _st(x)))
+        _chk("gap_forward", lib().shl_nn_gap_forward(_p(x), _p(y), B, C, H * W, _st(x)))
         ctx.shape = x.shape
         return y
 
     @staticmethod
     def backward(ctx, gy):
         B, C, H, W = ctx.shape
+        gy = gy.contiguous()
         gx = torch.empty(ctx.shape, dtype=torch.float32, device=gy.device)
-        _chk("gap_backward", lib().shl_nn_gap_backward(_p(gy.contiguous()), _p(gx), B, C, H * W, _st(gy)))
+        _chk("gap_backward", lib().shl_nn_gap_backward(_p(gy), _p(gx), B, C, H * W, _st(gy)))
         return gx
 
 
@@ -357,20 +363,22 @@ class _Linear(torch.autograd.Function):
     def forward(ctx, x, w, b):
         B, I = x.shape
         O = w.shape[0]
+        x, w, b = x.contiguous(), w.contiguous(), b.contiguous()
         y = torch.empty((B, O), dtype=torch.float32, device=x.device)
-        _chk("linear_forward", lib().shl_nn_linear_forward(_p(x.contiguous()), _p(w), _p(b), _p(y), B, I, O, _st(x)))
+        _chk("linear_forward", lib().shl_nn_linear_forward(_p(x), _p(w), _p(b), _p(y), B, I, O, _st(x)))
         ctx.save_for_backward(x, w)
         return y
 
     @staticmethod
     def backward(ctx, gy):
-        x, w = ctx.saved_tensors
+        x, w = ctx.saved_tensors                        # contiguous
+        gy = gy.contiguous()
         B, I = x.shape
         O = w.shape[0]
         gx = torch.empty_like(x)
         gw = torch.empty_like(w)
         gb = torch.empty(O, dtype=torch.float32, device=x.device)
-        _chk("linear_backward", lib().shl_nn_linear_backward(_p(x.contiguous()), _p(w), _p(gy.contiguous()), _p(gx),
+        _chk("linear_backward", lib().shl_nn_linear_backward(_p(x), _p(w), _p(gy), _p(gx),
                                                               _p(gw), _p(gb), B, I, O, _st(x)))
         return gx, gw, gb
 
@@ -387,8 +395,9 @@ class _Softplus(torch.autograd.Function):
     @staticmethod
     def backward(ctx, gy):
         (x,) = ctx.saved_tensors
+        gy = gy.contiguous()
         gx = torch.empty_like(x)
-        _chk("softplus_backward", lib().shl_nn_softplus_backward(_p(x), _p(gy.contiguous()), _p(gx), x.numel(), _st(x)))
+        _chk("softplus_backward", lib().shl_nn_softplus_backward(_p(x), _p(gy), _p(gx), x.numel(), _st(x)))
         return gx
 
 
@@ -401,6 +410,7 @@ class _Gate(torch.autograd.Function):
         assert c.dtype == torch.float32, "gate takes float32 coefficients"
         c = c.contiguous()
         delta = delta.contiguous()
+        scale = None if scale is None else scale.contiguous()
         B, K, H, W = c.shape
         y = torch.empty(c.shape, dtype=torch.float32, device=c.device)
         _chk("gate_forward", lib().shl_nn_gate_forward(_p(c), 0, _p(delta), _p(scale), K,
@@ -413,12 +423,13 @@ class _Gate(torch.autograd.Function):
     @staticmethod
     def backward(ctx, gy):
         c, delta = ctx.saved_tensors
+        gy = gy.contiguous()
         B, K, H, W = c.shape
         gc = torch.empty_like(c)
         gd = torch.empty_like(delta)
         ws = _ws(lib().shl_nn_gate_workspace_floats(B * K), c)
         _chk("gate_backward", lib().shl_nn_gate_backward(_p(c), _p(delta), _p(ctx.scale), K, ctx.tau,
-                                                          _p(gy.contiguous()), _p(gc), _p(gd), B * K,
+                                                          _p(gy), _p(gc), _p(gd), B * K,
                                                           H * W, _p(ws), _st(c)))
         return gc, gd, None, None
 
@@ -428,8 +439,12 @@ class _MaskMix(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, f_masked, mask_u8, f):
+        if f_masked.numel() != f.numel() or mask_u8.numel() != f.numel() or mask_u8.element_size() != 1:
+            raise ValueError("mask_mix takes f_masked and a mask of one byte per element of f")
+        # the kernels run through rows in order: transposed views are copied first
+        f_masked, mask_u8, f = f_masked.contiguous(), mask_u8.contiguous(), f.contiguous()
         u = torch.empty_like(f)
-        _chk("mask_mix", lib().shl_nn_mask_mix(_p(f_masked.contiguous()), _p(mask_u8), _p(f.contiguous()), _p(u),
+        _chk("mask_mix", lib().shl_nn_mask_mix(_p(f_masked), _p(mask_u8), _p(f), _p(u),
                                                 f.numel(), _st(f)))
         ctx.save_for_backward(mask_u8)
         return u
@@ -437,8 +452,9 @@ class _MaskMix(torch.autograd.Function):
     @staticmethod
     def backward(ctx, gu):
         (mask_u8,) = ctx.saved_tensors
+        gu = gu.contiguous()
         gf = torch.empty_like(gu)
-        _chk("mask_mix_backward", lib().shl_nn_mask_mix_backward(_p(mask_u8), _p(gu.contiguous()), _p(gf),
+        _chk("mask_mix_backward", lib().shl_nn_mask_mix_backward(_p(mask_u8), _p(gu), _p(gf),
                                                                   gu.numel(), _st(gu)))
         return None, None, gf
 
@@ -538,21 +554,24 @@ def mse(a, b):
 def scale_thresholds(d, scale, out):
     """out[t][b][k] = d[b][t][k] * scale[k] (no grad)."""
     B, T, K = d.shape
-    _chk("scale_thresholds", lib().shl_nn_scale_thresholds(_p(d.contiguous()), _p(scale), _p(out), B, T, K, _st(d)))
+    d, scale = d.contiguous(), scale.contiguous()
+    _chk("scale_thresholds", lib().shl_nn_scale_thresholds(_p(d), _p(scale), _p(out), B, T, K, _st(d)))
     return out
 
 
 def avgpool(x, f):
     B, C, H, W = x.shape
+    x = x.contiguous()
     y = torch.empty((B, C, H // f, W // f), dtype=torch.float32, device=x.device)
-    _chk("avgpool", lib().shl_nn_avgpool(_p(x.contiguous()), _p(y), B, C, H, W, f, _st(x)))
+    _chk("avgpool", lib().shl_nn_avgpool(_p(x), _p(y), B, C, H, W, f, _st(x)))
     return y
 
 
 def to_float(c):
     """bfloat16 -> float32 through the library's cast kernel (no grad)."""
+    c = c.contiguous()
     y = torch.empty(c.shape, dtype=torch.float32, device=c.device)
-    _chk("cast", lib().shl_nn_cast(_p(c.contiguous()), 1, _p(y), c.numel(), _st(c)))
+    _chk("cast", lib().shl_nn_cast(_p(c), 1, _p(y), c.numel(), _st(c)))
     return y
 
 
@@ -563,8 +582,9 @@ class _ToFloat(torch.autograd.Function):
 
     @staticmethod
     def backward(ctx, g):
+        g = g.contiguous()
         y = torch.empty(g.shape, dtype=torch.bfloat16, device=g.device)
-        _chk("cast", lib().shl_nn_cast(_p(g.contiguous()), 0, _p(y), g.numel(), _st(g)))
+        _chk("cast", lib().shl_nn_cast(_p(g), 0, _p(y), g.numel(), _st(g)))
         return y
 
 
@@ -719,6 +739,7 @@ class Adam:
         for p, m, v in zip(self.params, self.m, self.v):
             if p.grad is None:
                 continue
-            _chk("adam", lib().shl_nn_adam(_p(p), _p(p.grad.contiguous()), _p(m), _p(v), p.numel(),
+            g = p.grad.contiguous()
+            _chk("adam", lib().shl_nn_adam(_p(p), _p(g), _p(m), _p(v), p.numel(),
                                             self.lr, self.b1, self.b2, self.eps, self.step_count,
                                             _st(p)))
