@@ -67,9 +67,9 @@ size_t shl_nn_conv3x3_backward_weight_tc_workspace_floats(int B, int Ci, int Co,
 shl_status shl_nn_conv3x3_backward_weight_tc(const float* in, const float* gout, float* gw,
                                              float* gb, int B, int Ci, int Co, int H, int W,
                                              float* ws, void* stream);
-/* The same for layers of any number of input channels (up to 4096): groups of at
- * most 42 in one launch, their partials summed by one more.  Co, H, W and the
- * alignment as above; ws holds ..._wide_workspace_floats() floats (0: not
+/* The same for layers of any number of input channels: groups of at most 42, up to
+ * the number whose partials take 128 MB in one launch, summed by one more.  Co, H, W
+ * and the alignment as above; ws holds ..._wide_workspace_floats() floats (0: not
  * supported). */
 size_t shl_nn_conv3x3_backward_weight_tc_wide_workspace_floats(int B, int Ci, int Co, int H, int W);
 shl_status shl_nn_conv3x3_backward_weight_tc_wide(const float* in, const float* gout, float* gw,

@@ -386,13 +386,18 @@ __global__ void __launch_bounds__(CONV_THREADS, (ConvTcT<CG, NP>::MINB)) k_conv3
 // gw[o][i][dy][dx]; k_wgrad_reduce sums the partials in CTA order.
 // 3 Cin <= 128 rows hold at most WGRAD_CH input channels; wider layers run in groups
 // of them, one per blockIdx.y, which write disjoint entries of the same partials (the
-// bias ones come from the first group).
+// bias ones come from the first group).  A launch takes as many groups as keep its
+// partials within WGRAD_WS floats (128 MB), so that these do not grow with the layer
+// (1024 -> 96 channels: 540 MB in one launch).  Every layer of the networks here is one
+// launch; 4 x 128^2, 300 -> 96 channels, two launches in place of one: 211 -> 229 us.
 constexpr int WGRAD_CH = 42;
+constexpr size_t WGRAD_WS = (size_t)1 << 25;
 struct WgradTcArgs {
   const float* in;      // [B][Ctot][H][W]
   const float* gout;    // [B][Cout][H][W]
-  float* part;          // [gridDim.x][Cout * Ctot * 9 + Cout]: weight then bias partials
-  int B, Ctot, Cout, H, W;
+  float* part;          // [gridDim.x][Cout * Cslab * 9 + Cout]: weight then bias partials
+  int B, Ctot, Cslab;   // input channels of the layer, of this launch (`in` at its first)
+  int Cout, H, W;
   int rows_per_unit;    // output rows one CTA walks down per unit
   int Cin;              // channels of this CTA's group (set in the kernel)
 };
@@ -559,7 +564,7 @@ __global__ void __launch_bounds__(WgradTcT<NP>::THREADS, 1) k_wgrad_tc(const Wgr
   extern __shared__ __align__(128) uint8_t sm[];
   const int c0 = blockIdx.y * WGRAD_CH;       // the group's first input channel
   WgradTcArgs a = args;
-  a.Cin = min(WGRAD_CH, args.Ctot - c0);
+  a.Cin = min(WGRAD_CH, args.Cslab - c0);
   a.in += (size_t)c0 * a.H * a.W;
   uint8_t* As = sm;                           // SLOTS x [pg][128][8]
   uint8_t* Bs = sm + P::SLOTS * P::ABYTES;    // 2 x [pg][NP][8]
@@ -678,11 +683,11 @@ __global__ void __launch_bounds__(WgradTcT<NP>::THREADS, 1) k_wgrad_tc(const Wgr
     if (idx < a.Cout * P::PG) bred[idx] = bsum[k];
   }
   __syncthreads();
-  const size_t stride = (size_t)a.Cout * a.Ctot * 9 + a.Cout;
+  const size_t stride = (size_t)a.Cout * a.Cslab * 9 + a.Cout;
   if (c0 == 0 && tid < a.Cout) {   // items of channel o: idx = o * PG + pg
     float s = 0.f;
     for (int pg = 0; pg < P::PG; ++pg) s += bred[tid * P::PG + pg];
-    a.part[(size_t)blockIdx.x * stride + (size_t)a.Cout * a.Ctot * 9 + tid] = s;
+    a.part[(size_t)blockIdx.x * stride + (size_t)a.Cout * a.Cslab * 9 + tid] = s;
   }
   // epilogue (warps 0-3): lane r = dx * Cin + i, columns dy * NP + o
   if (!s_fail && warp < 4) {
@@ -702,7 +707,7 @@ __global__ void __launch_bounds__(WgradTcT<NP>::THREADS, 1) k_wgrad_tc(const Wgr
           for (int j = 0; j < 16; ++j) {
             const int o = 16 * q + j;
             if (o < a.Cout)
-              part[(((size_t)o * a.Ctot + c0 + i) * 3 + dy) * 3 + dx] =
+              part[(((size_t)o * a.Cslab + c0 + i) * 3 + dy) * 3 + dx] =
                   blockIdx.x < nunits ? __uint_as_float(acc[j]) : 0.f;
           }
         }
@@ -718,17 +723,19 @@ __global__ void __launch_bounds__(WgradTcT<NP>::THREADS, 1) k_wgrad_tc(const Wgr
                  : "memory");
 }
 
-// Sum the per-CTA partials in CTA order: entries e < nw are the weight
-// gradient, the next Cout the bias gradient (written only if gb != null).
+// Sum the per-CTA partials in CTA order: entries e < nw are the weight gradient of
+// the launch's channels (`row` = 9 Cslab per output channel, in rows of `pitch` = 9 Ctot),
+// the next Cout the bias gradient (written only if gb != null).
 __global__ void k_wgrad_reduce(const float* __restrict__ part, float* __restrict__ gw,
-                               float* __restrict__ gb, int nparts, int nw, int nb) {
+                               float* __restrict__ gb, int nparts, int nw, int nb, int row,
+                               size_t pitch) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   const int n = nw + nb;
   if (e >= n) return;
   float s = 0.f;
 #pragma unroll 8
   for (int c = 0; c < nparts; ++c) s += part[(size_t)c * n + e];   // eight loads in flight
-  if (e < nw) gw[e] = s;
+  if (e < nw) gw[e / row * pitch + e % row] = s;
   else if (gb) gb[e - nw] = s;
 }
 
@@ -747,6 +754,12 @@ void wgrad_plan(int B, int H, int W, int* grid, int* rows_per_unit) {
   *rows_per_unit = ru;
 }
 
+// Input channels of one launch of `grid` CTAs per group.
+int wgrad_slab(int grid, int Ci, int Co) {
+  const size_t groups = WGRAD_WS / ((size_t)grid * Co * 9 * WGRAD_CH);
+  return (int)std::min<size_t>(Ci, std::max<size_t>(1, groups) * WGRAD_CH);
+}
+
 template <int NP>
 cudaError_t launch_wgrad(const WgradTcArgs& a, int grid, cudaStream_t st) {
   using P = WgradTcT<NP>;
@@ -754,7 +767,7 @@ cudaError_t launch_wgrad(const WgradTcArgs& a, int grid, cudaStream_t st) {
   auto k = k_wgrad_tc<NP>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P::SMEM);
   if (e) return e;
-  k<<<dim3(grid, (a.Ctot + WGRAD_CH - 1) / WGRAD_CH), P::THREADS, P::SMEM, st>>>(a);
+  k<<<dim3(grid, (a.Cslab + WGRAD_CH - 1) / WGRAD_CH), P::THREADS, P::SMEM, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -1184,16 +1197,22 @@ static shl_status wgrad_run(const float* in, const float* gout, float* gw, float
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   int grid = 0, ru = 0;
   wgrad_plan(B, H, W, &grid, &ru);
-  const WgradTcArgs a{in, gout, ws, B, Ci, Co, H, W, ru, 0};
   const int np = round16(Co);          // 49..96 output channels: the 96-wide tile
-  cudaError_t e = np == 16 ? launch_wgrad<16>(a, grid, st)
-                : np == 32 ? launch_wgrad<32>(a, grid, st)
-                : np == 48 ? launch_wgrad<48>(a, grid, st)
-                           : launch_wgrad<96>(a, grid, st);
-  if (e == cudaSuccess) {
-    const int nw = Co * Ci * 9;
-    k_wgrad_reduce<<<(nw + Co + 127) / 128, 128, 0, st>>>(ws, gw, gb, grid, nw, Co);
+  const int slab = wgrad_slab(grid, Ci, Co);
+  cudaError_t e = cudaSuccess;
+  for (long long c0 = 0; c0 < Ci; c0 += slab) {
+    const int cs = (int)std::min<long long>(slab, Ci - c0);
+    const WgradTcArgs a{in + (size_t)c0 * H * W, gout, ws, B, Ci, cs, Co, H, W, ru, 0};
+    e = np == 16 ? launch_wgrad<16>(a, grid, st)
+      : np == 32 ? launch_wgrad<32>(a, grid, st)
+      : np == 48 ? launch_wgrad<48>(a, grid, st)
+                 : launch_wgrad<96>(a, grid, st);
+    if (e != cudaSuccess) break;
+    const int nw = Co * cs * 9;
+    k_wgrad_reduce<<<(nw + Co + 127) / 128, 128, 0, st>>>(ws, gw + c0 * 9, c0 ? nullptr : gb, grid,
+                                                          nw, Co, 9 * cs, (size_t)9 * Ci);
     e = cudaGetLastError();
+    if (e != cudaSuccess) break;
   }
   if (e != cudaSuccess) {
     g_tc_msg = "conv3x3_backward_weight_tc: launch failed";
@@ -1214,12 +1233,11 @@ shl_status shl_nn_conv3x3_backward_weight_tc(const float* in, const float* gout,
 }
 
 size_t shl_nn_conv3x3_backward_weight_tc_wide_workspace_floats(int B, int Ci, int Co, int H, int W) {
-  if (B < 1 || Ci < 1 || Ci > 4096 ||
-      !shl_nn_conv3x3_wgrad_tc_supported(std::min(Ci, WGRAD_CH), Co, H, W))
+  if (B < 1 || Ci < 1 || !shl_nn_conv3x3_wgrad_tc_supported(std::min(Ci, WGRAD_CH), Co, H, W))
     return 0;
   int grid = 0, ru = 0;
   wgrad_plan(B, H, W, &grid, &ru);
-  return (size_t)grid * ((size_t)Co * Ci * 9 + Co);
+  return (size_t)grid * ((size_t)Co * wgrad_slab(grid, Ci, Co) * 9 + Co);
 }
 
 shl_status shl_nn_conv3x3_backward_weight_tc_wide(const float* in, const float* gout, float* gw,
