@@ -490,11 +490,13 @@ shl_status decompose_impl(const shl_bank* b, shl::InMode mode, const float* x,
   return SHL_OK;
 }
 
+constexpr int MAX_GRID_Y = 65535;   // planes (or images) that one launch can index by blockIdx.y
+
 // Reconstruction-style chunks (whole images when the staging area holds K
-// subbands, else filter ranges inside one image), shared by reconstruct_impl
-// and shrink_impl.
+// subbands, at most MAX_GRID_Y of them, else filter ranges inside one image),
+// shared by the reconstructions and the shrinks.
 int next_chunk(int s0, int total, int S, int K) {
-  if (S >= K) return std::min((S / K) * K, total - s0);
+  if (S >= K) return std::min(std::min(S / K, MAX_GRID_Y) * K, total - s0);
   const int img_end = (s0 / K + 1) * K;
   return std::min(S, img_end - s0);
 }
@@ -667,9 +669,9 @@ cudaError_t gen_image_spectra(const shl_bank* b, shl::InMode mode, const float* 
                            fest, nullptr, X, N, batch, st);
   }
   if (e) return e;
-  for (int b0 = 0; b0 < batch; b0 += 65535) {
+  for (int b0 = 0; b0 < batch; b0 += MAX_GRID_Y) {
     Launch L_("gen_cols_fwd_image", st);
-    e = G::launch_cols_fwd(b->planN, X + (size_t)b0 * N * Mh, Mh, std::min(65535, batch - b0), st);
+    e = G::launch_cols_fwd(b->planN, X + (size_t)b0 * N * Mh, Mh, std::min(MAX_GRID_Y, batch - b0), st);
     if (e) return e;
   }
   return cudaSuccess;
@@ -688,7 +690,7 @@ cudaError_t gen_decompose(const shl_bank* b, shl::InMode mode, const float* x,
   const int total = batch * K;
   const size_t esz = dtype == SHL_BF16 ? 2 : 4;
   const float scale = (float)(1.0 / (double(N) * M));
-  S = std::min(S, 65535);
+  S = std::min(S, MAX_GRID_Y);
   for (int s0 = 0; s0 < total; s0 += S) {
     const int Sc = std::min(S, total - s0);
     {
@@ -753,7 +755,7 @@ cudaError_t gen_shrink(const shl_bank* b, const float* x, const unsigned char* m
   cudaError_t e = gen_image_spectra(b, mask ? shl::IN_MASKED : shl::IN_F32, x, mask, fest, batch,
                                     X, st);
   if (e) return e;
-  const int total = batch * K, S = stage_subbands(b);
+  const int total = batch * K, S = std::min(stage_subbands(b), MAX_GRID_Y);
   for (int s0 = 0; s0 < total;) {
     const int Sc = next_chunk(s0, total, S, K);
     {
