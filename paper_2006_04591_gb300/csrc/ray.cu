@@ -22,6 +22,7 @@
 #include <cmath>
 #include <cstdint>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/shearlet_ray.h"
@@ -177,8 +178,8 @@ __global__ void __launch_bounds__(FWD_BINS) k_ray_forward(const float* __restric
 
 // ---------------------------------------------------------------- adjoint
 // Pixel (t, k) of angle a receives every bin d with |u(d, t) - k| < 1, with the
-// hat weight 1 - |u - k|: exactly the forward's 1 - w1 or w1, since u - k and
-// the difference from 1 on the far side are exact in float32.  The bins start at
+// forward's own weight, rounding included (hat_weight), so that the two are exact
+// transposes.  The bins start at
 // the one below the fractional bin of u = k - 1; ADJ_MARGIN covers the rounding
 // of that bin (below 0.01 over the accepted sizes).  What bounds it: the
 // bins' reads through L1, shared by nothing but the four images' position, weights
@@ -187,6 +188,17 @@ __global__ void __launch_bounds__(FWD_BINS) k_ray_forward(const float* __restric
 // images of 128 x 128 at 30 angles: 96 and 33 us (forward 107 and 45 us).
 constexpr float ADJ_MARGIN = 0.05f;
 constexpr int ADJ_PIX = 2;         // pixels per thread, 8 rows apart
+
+// What the forward's sample at u gives pixel k (zero or less: nothing): 1 - (u - k) above
+// it, u - (k - 1) below.  Both are 1 - |u - k| to the last bit, as u - k is exact or the
+// sum rounds once, except at k = 1: for 0 < u < 1/2 u - 1 is not a float32 and would
+// round twice.  EDGE: CTAs that may hold k = 1, those of the first row and column of
+// the image (8 x 700^2, 90 angles: 234 us without it, 237 us so, 256 us in all CTAs; 8 x
+// 512^2, 180 angles, which is one wave: 277, 296 and 301 us).
+template <bool EDGE>
+__device__ __forceinline__ float hat_weight(float u, float k) {
+  return EDGE ? fminf(u - (k - 1.f), 1.f - (u - k)) : __saturatef(1.f - fabsf(u - k));
+}
 
 template <int NB>
 __global__ void __launch_bounds__(256) k_ray_adjoint(const float* __restrict__ sino,
@@ -203,39 +215,43 @@ __global__ void __launch_bounds__(256) k_ray_adjoint(const float* __restrict__ s
   for (int x = 0; x < ADJ_PIX; ++x)
 #pragma unroll
     for (int b = 0; b < NB; ++b) acc[x][b] = 0.f;
-  for (int a = 0; a < A; ++a) {
-    const AngleParam q = load_angle(prm + a);
-    const float first = fabsf(q.inv_a) + (ADJ_MARGIN + 0.5f);
-    const int row = a * D;
+  auto angles = [&](auto edge) {
+    for (int a = 0; a < A; ++a) {
+      const AngleParam q = load_angle(prm + a);
+      const float first = fabsf(q.inv_a) + (ADJ_MARGIN + 0.5f);
+      const int row = a * D;
 #pragma unroll
-    for (int x = 0; x < ADJ_PIX; ++x) {
-      const int i = i0 + 8 * x;
-      const float t = (float)(q.by_rows ? i : j), k = (float)(q.by_rows ? j : i);
-      const float base = fmaf(q.B, t, q.C);
-      int lo;
-      const float flo = round_near(fminf(fmaxf((k - base) * q.inv_a - first, -1e6f), 1e6f), &lo);
-      float sa[NB];
+      for (int x = 0; x < ADJ_PIX; ++x) {
+        const int i = i0 + 8 * x;
+        const float t = (float)(q.by_rows ? i : j), k = (float)(q.by_rows ? j : i);
+        const float base = fmaf(q.B, t, q.C);
+        int lo;
+        const float flo = round_near(fminf(fmaxf((k - base) * q.inv_a - first, -1e6f), 1e6f), &lo);
+        float sa[NB];
 #pragma unroll
-      for (int b = 0; b < NB; ++b) sa[b] = 0.f;
-      auto bin = [&](int m) {
-        const float w = __saturatef(1.f - fabsf(fmaf(q.A, flo + (float)m, base) - k));
-        if (w > 0.f) {               // a bin outside the hat is not read into the sum
+        for (int b = 0; b < NB; ++b) sa[b] = 0.f;
+        auto bin = [&](int m) {
+          const float w = hat_weight<decltype(edge)::value>(fmaf(q.A, flo + (float)m, base), k);
+          if (w > 0.f) {               // a bin outside the hat is not read into the sum
 #pragma unroll
-          for (int b = 0; b < NB; ++b) sa[b] = fmaf(w, __ldg(p[b] + (row + lo + m)), sa[b]);
+            for (int b = 0; b < NB; ++b) sa[b] = fmaf(w, __ldg(p[b] + (row + lo + m)), sa[b]);
+          }
+        };
+        if (lo >= 0 && lo + q.bins <= D) {
+          bin(0);
+          bin(1);
+          if (q.bins > 2) bin(2);
+          for (int m = 3; m < q.bins; ++m) bin(m);
+        } else {
+          for (int m = max(0, -lo); m < q.bins && lo + m < D; ++m) bin(m);
         }
-      };
-      if (lo >= 0 && lo + q.bins <= D) {
-        bin(0);
-        bin(1);
-        if (q.bins > 2) bin(2);
-        for (int m = 3; m < q.bins; ++m) bin(m);
-      } else {
-        for (int m = max(0, -lo); m < q.bins && lo + m < D; ++m) bin(m);
-      }
 #pragma unroll
-      for (int b = 0; b < NB; ++b) acc[x][b] = fmaf(sa[b], q.w, acc[x][b]);
+        for (int b = 0; b < NB; ++b) acc[x][b] = fmaf(sa[b], q.w, acc[x][b]);
+      }
     }
-  }
+  };
+  if (blockIdx.x > 0 && blockIdx.y > 0) angles(std::false_type{});
+  else angles(std::true_type{});
 #pragma unroll
   for (int x = 0; x < ADJ_PIX; ++x)
 #pragma unroll
@@ -246,7 +262,8 @@ __global__ void __launch_bounds__(256) k_ray_adjoint(const float* __restrict__ s
 
 // The same with the bins that a tile of 32 x 32 pixels can receive staged in shared
 // memory, images interleaved: one NB-wide read per bin in place of NB gathers
-// through L1.  Chunks of `ac` angles, W bins each; lo_of the first staged bin.
+// through L1 (measured as above 527 -> 277 us, 296 us with the exact weights).  Chunks
+// of `ac` angles, W bins each, from bin s_lo on.
 constexpr int ADJ_TILE_PIX = 4;    // pixels per thread, 8 rows apart
 constexpr int ADJ_CHUNK = 16;      // most angles staged at a time
 constexpr size_t ADJ_SMEM = 48 * 1024;
@@ -296,38 +313,42 @@ __global__ void __launch_bounds__(256) k_ray_adjoint_tile(const float* __restric
       S[idx] = v;
     }
     __syncthreads();
-    for (int a = 0; a < na; ++a) {
-      const AngleParam q = load_angle(prm + a0 + a);
-      const float first = fabsf(q.inv_a) + (ADJ_MARGIN + 0.5f);
-      const int lo0 = s_lo[a];
-      const Vec<NB>* s = S + a * W;
+    auto angles = [&](auto edge) {
+      for (int a = 0; a < na; ++a) {
+        const AngleParam q = load_angle(prm + a0 + a);
+        const float first = fabsf(q.inv_a) + (ADJ_MARGIN + 0.5f);
+        const int lo0 = s_lo[a];
+        const Vec<NB>* s = S + a * W;
 #pragma unroll
-      for (int x = 0; x < ADJ_TILE_PIX; ++x) {
-        const int i = i0 + 8 * x;
-        const float t = (float)(q.by_rows ? i : j), k = (float)(q.by_rows ? j : i);
-        const float base = fmaf(q.B, t, q.C);
-        int lo;
-        const float flo = round_near(fminf(fmaxf((k - base) * q.inv_a - first, -1e6f), 1e6f), &lo);
-        const Vec<NB>* r = s + min(max(lo - lo0, 0), W - q.bins);
-        float sa[NB];
+        for (int x = 0; x < ADJ_TILE_PIX; ++x) {
+          const int i = i0 + 8 * x;
+          const float t = (float)(q.by_rows ? i : j), k = (float)(q.by_rows ? j : i);
+          const float base = fmaf(q.B, t, q.C);
+          int lo;
+          const float flo = round_near(fminf(fmaxf((k - base) * q.inv_a - first, -1e6f), 1e6f), &lo);
+          const Vec<NB>* r = s + min(max(lo - lo0, 0), W - q.bins);
+          float sa[NB];
 #pragma unroll
-        for (int b = 0; b < NB; ++b) sa[b] = 0.f;
-        auto bin = [&](int m) {
-          const float w = __saturatef(1.f - fabsf(fmaf(q.A, flo + (float)m, base) - k));
-          const Vec<NB> v = r[m];
-          if (w > 0.f) {               // a bin outside the hat does not enter the sum
+          for (int b = 0; b < NB; ++b) sa[b] = 0.f;
+          auto bin = [&](int m) {
+            const float w = hat_weight<decltype(edge)::value>(fmaf(q.A, flo + (float)m, base), k);
+            const Vec<NB> v = r[m];
+            if (w > 0.f) {               // a bin outside the hat does not enter the sum
 #pragma unroll
-            for (int b = 0; b < NB; ++b) sa[b] = fmaf(w, v.v[b], sa[b]);
-          }
-        };
-        bin(0);
-        bin(1);
-        if (q.bins > 2) bin(2);
-        for (int m = 3; m < q.bins; ++m) bin(m);
+              for (int b = 0; b < NB; ++b) sa[b] = fmaf(w, v.v[b], sa[b]);
+            }
+          };
+          bin(0);
+          bin(1);
+          if (q.bins > 2) bin(2);
+          for (int m = 3; m < q.bins; ++m) bin(m);
 #pragma unroll
-        for (int b = 0; b < NB; ++b) acc[x][b] = fmaf(sa[b], q.w, acc[x][b]);
+          for (int b = 0; b < NB; ++b) acc[x][b] = fmaf(sa[b], q.w, acc[x][b]);
+        }
       }
-    }
+    };
+    if (j0 > 0 && r0 > 0) angles(std::false_type{});
+    else angles(std::true_type{});
   }
 #pragma unroll
   for (int x = 0; x < ADJ_TILE_PIX; ++x)
