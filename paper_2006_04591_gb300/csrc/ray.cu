@@ -77,11 +77,20 @@ template <> struct __align__(16) Vec<4> { float v[4]; };
 // the same, interleaving NB images shares the position and the weights between
 // them, and two neighbouring angles share one staging.  Measured at 8 images of
 // 512 x 512, 180 angles, 725 bins: 1402 us with one thread per ray, 338 us so (one
-// image: 239 and 187 us).
+// image: 239 and 121 us).
+//
+// With one or two images per CTA it waits for the staged pixels instead: a thread takes
+// its share of a staging in batches of up to FWD_WORDS loads, and launches of fewer CTAs
+// than SMs take one angle per CTA.  600 x 600, 60 angles, 849 bins, one and two images:
+// 145 and 170 us with one thread per ray, 213 and 216 us without either, 112 and 143 us
+// so; one image of 700 x 700, 180 angles, 128 bins: 190, 443 and 170 us.  (Four images:
+// batches of four pixels 338 -> 315 us at the size above, but 39 -> 46 us at 130 images
+// of 96 x 96; not taken.)
 constexpr int FWD_BINS = 256;      // bins (threads) per CTA
 constexpr int FWD_ANGLES = 2;      // most angles per CTA
 constexpr int FWD_ROWS = 8;        // most samples t staged at a time
 constexpr size_t FWD_SMEM = 56 * 1024;   // four CTAs per SM
+constexpr int FWD_WORDS = 16;      // most words a thread loads before it stores them
 
 struct AngleGroup { int a0, na; };   // neighbouring angles of one kind
 
@@ -94,7 +103,7 @@ __global__ void __launch_bounds__(FWD_BINS) k_ray_forward(const float* __restric
   extern __shared__ __align__(16) unsigned char smem[];
   Vec<NB>* S = reinterpret_cast<Vec<NB>*>(smem);     // [T][pitch]
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const AngleGroup grp = groups[blockIdx.y];
+  const AngleGroup grp = groups ? groups[blockIdx.y] : AngleGroup{(int)blockIdx.y, 1};
   const int d_lo = blockIdx.x * FWD_BINS, d_hi = min(D - 1, d_lo + FWD_BINS - 1);
   const int d = d_lo + tid, b0 = blockIdx.z * NB;
   const float df = (float)min(d, d_hi);
@@ -128,7 +137,40 @@ __global__ void __launch_bounds__(FWD_BINS) k_ray_forward(const float* __restric
     const int k_hi = min(n + 1, (int)floorf(fminf(hi, (float)(n + 4))) + 1);
     const int width = min(k_hi - k_lo + 1, pitch);
     __syncthreads();                                 // the earlier rows have been read
-    if (by_rows) {
+    // sample row tt, pixels x0, x0 + 32, ..: pixel k of sample t is at k sk + t st.  U loads
+    // per image in flight, halved while the rest of the row needs no more than that.
+    auto stage = [&](int tt, int x0, int sk, int st) {
+      auto batch = [&](int x, auto uc) {
+        constexpr int U = decltype(uc)::value;
+        const int at = (k_lo + x) * sk + (t0 + tt) * st;
+        Vec<NB> v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int k = k_lo + x + 32 * u;
+          const bool in = k >= 0 && k < n && x + 32 * u < width;
+#pragma unroll
+          for (int b = 0; b < NB; ++b) v[u].v[b] = in ? __ldg(f[b] + (at + 32 * u * sk)) : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (x + 32 * u < width) S[tt * pitch + x + 32 * u] = v[u];
+      };
+      constexpr int U = FWD_WORDS / NB;
+      for (int x = 0; x < width; x += 32 * U) {
+        const int rest = (width - x + 31) / 32;
+        if (rest > U / 2) batch(x0 + x, std::integral_constant<int, U>{});
+        else if (rest > U / 4) batch(x0 + x, std::integral_constant<int, U / 2>{});
+        else batch(x0 + x, std::integral_constant<int, (U > 4 ? U / 4 : 1)>{});
+      }
+    };
+    if constexpr (NB < 4) {
+      if (by_rows) {
+        for (int tt = warp; tt < tn; tt += FWD_BINS / 32) stage(tt, lane, 1, n);
+      } else {                                       // FWD_ROWS consecutive columns of a pixel row
+        const int tt = lane & (FWD_ROWS - 1);
+        if (tt < tn) stage(tt, warp * (32 / FWD_ROWS) + lane / FWD_ROWS, n, 1);
+      }
+    } else if (by_rows) {
       for (int tt = warp; tt < tn; tt += FWD_BINS / 32)
         for (int x = lane; x < width; x += 32) {
           const int k = k_lo + x;
@@ -400,9 +442,11 @@ cudaError_t forward_nb(const shl_ray* op, const float* img, int batch, float* si
   if (smem > 48 * 1024)
     e = cudaFuncSetAttribute(k_ray_forward<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e) return e;
-  const dim3 grid((op->D + FWD_BINS - 1) / FWD_BINS, op->ngrp, (batch + NB - 1) / NB);
-  k_ray_forward<NB><<<grid, FWD_BINS, smem, st>>>(img, sino, op->dPrm, op->dGrp, op->n, op->A, op->D,
-                                                  batch, T, pitch);
+  dim3 grid((op->D + FWD_BINS - 1) / FWD_BINS, op->ngrp, (batch + NB - 1) / NB);
+  const bool single_angles = (long long)grid.x * grid.y * grid.z < op->sms;
+  if (single_angles) grid.y = op->A;
+  k_ray_forward<NB><<<grid, FWD_BINS, smem, st>>>(img, sino, op->dPrm, single_angles ? nullptr : op->dGrp,
+                                                  op->n, op->A, op->D, batch, T, pitch);
   return cudaGetLastError();
 }
 
