@@ -229,7 +229,10 @@ __global__ void __launch_bounds__(FWD_BINS) k_ray_forward(const float* __restric
 // per pixel and image (a floor and a compare per candidate bin), 527 us so; 32
 // images of 128 x 128 at 30 angles: 96 and 33 us (forward 107 and 45 us).
 constexpr float ADJ_MARGIN = 0.05f;
-constexpr int ADJ_PIX = 2;         // pixels per thread, 8 rows apart
+constexpr int ADJ_PIX = 2;         // pixels per thread, 8 rows apart; one where that leaves
+                                   // SMs without two CTAs (16^2, 8 angles, 2000
+                                   // bins: 184 -> 117 us, 158 us with one thread per pixel;
+                                   // 256^2, 180 angles, one image: 121 -> 92 us)
 
 // What the forward's sample at u gives pixel k (zero or less: nothing): 1 - (u - k) above
 // it, u - (k - 1) below.  Both are 1 - |u - k| to the last bit, as u - k is exact or the
@@ -242,19 +245,19 @@ __device__ __forceinline__ float hat_weight(float u, float k) {
   return EDGE ? fminf(u - (k - 1.f), 1.f - (u - k)) : __saturatef(1.f - fabsf(u - k));
 }
 
-template <int NB>
+template <int NB, int PIX>
 __global__ void __launch_bounds__(256) k_ray_adjoint(const float* __restrict__ sino,
                                                      float* __restrict__ img,
                                                      const AngleParam* __restrict__ prm, int n,
                                                      int A, int D, int B) {
   const int j = blockIdx.x * 32 + (threadIdx.x & 31);
-  const int i0 = blockIdx.y * (8 * ADJ_PIX) + (threadIdx.x >> 5), b0 = blockIdx.z * NB;
+  const int i0 = blockIdx.y * (8 * PIX) + (threadIdx.x >> 5), b0 = blockIdx.z * NB;
   const float* p[NB];
 #pragma unroll
   for (int b = 0; b < NB; ++b) p[b] = sino + (size_t)min(b0 + b, B - 1) * A * D;
-  float acc[ADJ_PIX][NB];
+  float acc[PIX][NB];
 #pragma unroll
-  for (int x = 0; x < ADJ_PIX; ++x)
+  for (int x = 0; x < PIX; ++x)
 #pragma unroll
     for (int b = 0; b < NB; ++b) acc[x][b] = 0.f;
   auto angles = [&](auto edge) {
@@ -263,7 +266,7 @@ __global__ void __launch_bounds__(256) k_ray_adjoint(const float* __restrict__ s
       const float first = fabsf(q.inv_a) + (ADJ_MARGIN + 0.5f);
       const int row = a * D;
 #pragma unroll
-      for (int x = 0; x < ADJ_PIX; ++x) {
+      for (int x = 0; x < PIX; ++x) {
         const int i = i0 + 8 * x;
         const float t = (float)(q.by_rows ? i : j), k = (float)(q.by_rows ? j : i);
         const float base = fmaf(q.B, t, q.C);
@@ -295,7 +298,7 @@ __global__ void __launch_bounds__(256) k_ray_adjoint(const float* __restrict__ s
   if (blockIdx.x > 0 && blockIdx.y > 0) angles(std::false_type{});
   else angles(std::true_type{});
 #pragma unroll
-  for (int x = 0; x < ADJ_PIX; ++x)
+  for (int x = 0; x < PIX; ++x)
 #pragma unroll
     for (int b = 0; b < NB; ++b)
       if (j < n && i0 + 8 * x < n && b0 + b < B)
@@ -464,8 +467,13 @@ cudaError_t adjoint_nb(const shl_ray* op, const float* sino, int batch, float* i
         sino, img, op->dPrm, op->n, op->A, op->D, batch, W, ac);
     return cudaGetLastError();
   }
-  const dim3 grid((op->n + 31) / 32, (op->n + 8 * ADJ_PIX - 1) / (8 * ADJ_PIX), (batch + NB - 1) / NB);
-  k_ray_adjoint<NB><<<grid, 256, 0, st>>>(sino, img, op->dPrm, op->n, op->A, op->D, batch);
+  dim3 grid((op->n + 31) / 32, (op->n + 8 * ADJ_PIX - 1) / (8 * ADJ_PIX), (batch + NB - 1) / NB);
+  if (NB == 1 && (long long)grid.x * grid.y * grid.z < 2LL * op->sms) {   // NB > 1: never so few
+    grid.y = (op->n + 7) / 8;
+    k_ray_adjoint<1, 1><<<grid, 256, 0, st>>>(sino, img, op->dPrm, op->n, op->A, op->D, batch);
+  } else {
+    k_ray_adjoint<NB, ADJ_PIX><<<grid, 256, 0, st>>>(sino, img, op->dPrm, op->n, op->A, op->D, batch);
+  }
   return cudaGetLastError();
 }
 
