@@ -715,7 +715,14 @@ constexpr int DEC_FPG = 4;
 
 // One lane group: kx line `kx` of the chunk subbands sl0..sl1-1 (global
 // subband s0 + sl, image s / K, filter s mod K) into out[sl][kx][:].
-template <int LOG_N, bool S16 = false>
+//
+// RELOAD (32 values per lane, float32): the spectrum line is read again for every filter
+// (from L2), which leaves two CTAs per SM where holding it leaves one.  For launches that
+// fill more than one CTA per SM (lines_t): 1 x 1024^2, K = 17, 1.07 times and 4 x 1024^2,
+// K = 49, 249 -> 215 us; smaller ones only wait for the extra loads (1 x 1024 x 64, K = 17:
+// 25.1 us held, 26.2 us reloaded).  2048-point lines are never faster so (1 x 2048 x 512:
+// 83.9 and 84.4 us; with one CTA per SM 88 us).
+template <int LOG_N, bool S16 = false, bool RELOAD = false>
 __device__ __forceinline__ void dec_group(const float2* X, void* out, const float* Gall,
                                           const float* invW, float scale, int Mh, int K, int s0,
                                           int sl0, int sl1, int kx, float2* line, const float2* twl,
@@ -724,11 +731,7 @@ __device__ __forceinline__ void dec_group(const float2* X, void* out, const floa
   using P = LinesT<LOG_N>;
   constexpr int T = P::T, R = P::R, N = P::N;
   const float* W = invW ? invW + (size_t)kx * N : nullptr;
-  if constexpr (R >= 32 && !S16) {
-    // 32 values per lane: reading the spectrum line again for every filter (from L2)
-    // leaves two CTAs per SM where holding it left one (4 x 1024^2: 249 -> 215 us;
-    // at 16 values per lane a third CTA gains nothing; the bfloat16 form keeps its
-    // rounding, see dft_reg)
+  if constexpr (RELOAD) {
     for (int sl = sl0; sl < sl1; ++sl) {
       const int s = s0 + sl, b = s / K, i = s - b * K;
       const float2* Xp = X + ((size_t)b * Mh + kx) * N;
@@ -801,8 +804,8 @@ __device__ __forceinline__ void dec_group(const float2* X, void* out, const floa
   }
 }
 
-template <int LOG_N, bool S16>
-__global__ void __launch_bounds__(256, LOG_N == 10 && !S16 ? 2 : 1) k_dec_lines(LinesArgs a) {
+template <int LOG_N, bool S16, bool RELOAD = false>
+__global__ void __launch_bounds__(256, RELOAD ? 2 : 1) k_dec_lines(LinesArgs a) {
   using P = LinesT<LOG_N>;
   constexpr int T = P::T, R = P::R, N = P::N;
   extern __shared__ float2 smem[];
@@ -818,7 +821,7 @@ __global__ void __launch_bounds__(256, LOG_N == 10 && !S16 ? 2 : 1) k_dec_lines(
   for (int q = blockIdx.x * P::NG + g; q < items; q += gridDim.x * P::NG) {
     const int m = q / a.Mh, kx = q - m * a.Mh;
     const int sl0 = m * DEC_FPG, sl1 = min(S, sl0 + DEC_FPG);
-    dec_group<LOG_N, S16>(a.data, a.out, a.G, a.invW, a.scale, a.Mh, a.K, a.s0, sl0, sl1, kx, line,
+    dec_group<LOG_N, S16, RELOAD>(a.data, a.out, a.G, a.invW, a.scale, a.Mh, a.K, a.s0, sl0, sl1, kx, line,
                           twl, j, g, a.nimg, S);
   }
 }
@@ -1207,6 +1210,10 @@ static cudaError_t shrink_t(const RowsShrinkArgs& a, cudaStream_t st) {
 
 constexpr int MAX_DEVICES = 16;   // devices whose occupancy is kept
 
+// Lengths whose float32 decomposition has the reloading form (dec_group).
+template <int LOG_N>
+__host__ __device__ constexpr bool dec_reload() { return LOG_N == 10; }
+
 template <int LOG_N>
 static cudaError_t lines_t(int mode, const LinesArgs& a, const RecLinesArgs& ra, int grid_y,
                            cudaStream_t st) {
@@ -1218,8 +1225,9 @@ static cudaError_t lines_t(int mode, const LinesArgs& a, const RecLinesArgs& ra,
     const size_t sm = P::SMEM_LINES + P::TWB;
     // persistent grid-stride: exactly the CTAs that fit at once, so that no
     // partial last wave is left; the count is asked for once per kernel and device
-    const int which = mode == 0 ? 0 : a.s16 ? 1 : 2;
-    static std::atomic<int> cached[3][MAX_DEVICES];
+    const int ctas = (work + P::NG - 1) / P::NG;
+    const int which = mode == 0 ? 0 : a.s16 ? 1 : dec_reload<LOG_N>() && ctas > sm_count() ? 3 : 2;
+    static std::atomic<int> cached[4][MAX_DEVICES];
     int dev = 0;
     if ((e = cudaGetDevice(&dev))) return e;
     int per_sm = dev < MAX_DEVICES ? cached[which][dev].load(std::memory_order_relaxed) : 0;
@@ -1230,13 +1238,17 @@ static cudaError_t lines_t(int mode, const LinesArgs& a, const RecLinesArgs& ra,
       if (!r && dev < MAX_DEVICES) cached[which][dev].store(per_sm, std::memory_order_relaxed);
       return r;
     };
-    e = which == 0 ? ask(k_lines_fwd<LOG_N>) : which == 1 ? ask(k_dec_lines<LOG_N, true>)
-                                                          : ask(k_dec_lines<LOG_N, false>);
+    auto run = [&](auto kernel) -> cudaError_t {
+      cudaError_t r = ask(kernel);
+      if (r) return r;
+      kernel<<<std::max(1, std::min(ctas, std::max(per_sm, 1) * sm_count())), P::THREADS, sm, st>>>(a);
+      return cudaSuccess;
+    };
+    constexpr bool RL = dec_reload<LOG_N>();
+    e = which == 0 ? run(k_lines_fwd<LOG_N>)
+      : which == 1 ? run(k_dec_lines<LOG_N, true>)
+      : which == 2 ? run(k_dec_lines<LOG_N, false>) : run(k_dec_lines<LOG_N, false, RL>);
     if (e) return e;
-    const int grid = std::max(1, std::min((work + P::NG - 1) / P::NG, std::max(per_sm, 1) * sm_count()));
-    if (mode == 0) k_lines_fwd<LOG_N><<<grid, P::THREADS, sm, st>>>(a);
-    else if (a.s16) k_dec_lines<LOG_N, true><<<grid, P::THREADS, sm, st>>>(a);
-    else k_dec_lines<LOG_N, false><<<grid, P::THREADS, sm, st>>>(a);
   } else {
     using Q = LinesT<LOG_N, true>;
     const size_t sm = Q::SMEM_LINES + sizeof(float2) * (size_t)Q::NG * Q::N + Q::TWB;
