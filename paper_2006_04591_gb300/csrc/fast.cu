@@ -684,6 +684,12 @@ struct LinesArgs {
   int s16;                   // DEC: bfloat16 staging (the bfloat16 decomposition)
 };
 
+// Reconstruction and float32 decomposition columns use packed additions from 128 points
+// on (there and back at 128 x 128, 64 images: 1.02 times); at 64 and 32 they cost 1 %
+// (reconstruction of 64 x 1024, 64 images, K = 17: 531 -> 536 us).
+template <int LOG_N>
+__host__ __device__ constexpr bool lines_packed() { return LOG_N >= 7; }
+
 template <int LOG_N>
 __global__ void __launch_bounds__(256) k_lines_fwd(LinesArgs a) {
   using P = LinesT<LOG_N>;
@@ -745,7 +751,8 @@ __device__ __forceinline__ void dec_group(const float2* X, void* out, const floa
         if (W) gv *= __ldg(W + j + u * T);
         v[u] = ok ? cscale(Xp[j + u * T], gv) : make_float2(0.f, 0.f);
       }
-      line_fft_any<N, R, +1, !S16>(v, line, j, 1 + g, twl, twl + LineTw<N, R>::WORDS);
+      line_fft_any<N, R, +1, (!S16 && lines_packed<LOG_N>())>(v, line, j, 1 + g, twl,
+                                                               twl + LineTw<N, R>::WORDS);
       if (!SHL_IN((size_t)sl * Mh + kx, (size_t)nstage * Mh, CHK_DEC_OUT)) continue;
       float2* o = static_cast<float2*>(out) + ((size_t)sl * Mh + kx) * N;
 #pragma unroll
@@ -789,7 +796,8 @@ __device__ __forceinline__ void dec_group(const float2* X, void* out, const floa
       if (W) gv *= __ldg(W + j + u * T);
       v[u] = cscale(Xl[u], gv);
     }
-    line_fft_any<N, R, +1, !S16>(v, line, j, 1 + g, twl, twl + LineTw<N, R>::WORDS);
+    line_fft_any<N, R, +1, (!S16 && lines_packed<LOG_N>())>(v, line, j, 1 + g, twl,
+                                                               twl + LineTw<N, R>::WORDS);
     if (SHL_IN((size_t)sl * Mh + kx, (size_t)nstage * Mh, CHK_DEC_OUT)) {
       if constexpr (S16) {
         __nv_bfloat162* o = static_cast<__nv_bfloat162*>(out) + ((size_t)sl * Mh + kx) * N;
@@ -880,7 +888,7 @@ __global__ void __launch_bounds__(256, LinesT<LOG_N, true>::R >= 32 ? 1 : 2) k_r
     group_sync<T>(1 + g);                   // line read before it is overwritten
     if (s + NG < s_end) fetch(s + NG);
     cp_async_commit();
-    line_fft_any<N, R, -1, true>(v, line, j, 1 + g, twl, twb);
+    line_fft_any<N, R, -1, lines_packed<LOG_N>()>(v, line, j, 1 + g, twl, twb);
 #pragma unroll
     for (int u = 0; u < R; ++u) {
       const float gv = gok ? __ldg(G + j + u * T) : 0.f;
@@ -913,7 +921,7 @@ __global__ void __launch_bounds__(256, LinesT<LOG_N, true>::R >= 32 ? 1 : 2) k_r
     float2 v[R];
 #pragma unroll
     for (int u = 0; u < R; ++u) v[u] = red[j + u * T];
-    line_fft_any<N, R, +1, true>(v, line, j, 1, twl, twb);
+    line_fft_any<N, R, +1, lines_packed<LOG_N>()>(v, line, j, 1, twl, twb);
 #pragma unroll
     for (int u = 0; u < R; ++u) A[j + u * T] = v[u];
   }
