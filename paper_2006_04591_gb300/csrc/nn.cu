@@ -208,11 +208,15 @@ __global__ void k_conv_wgrad_reduce(const float* __restrict__ partial, float* __
 // What bounds these: DRAM.  A thread has EW_U float4 of each operand in flight
 // before it uses the first (one kept the copy rate at 70-80 %).  Measured at
 // 32 x 32 x 256^2 (268 MB per operand): PReLU forward 103 -> 77 us (7.0 TB/s),
-// backward 139 -> 121 us (6.7 TB/s).
+// backward 139 -> 121 us (6.7 TB/s).  Below EW_FEW float4 four in flight leave too few
+// CTAs and a thread takes one: backward at 174,720 elements 4.2 us with one, 4.6 us with
+// four; at 327,680 4.3 and 4.2 us.
 constexpr int EW_U = 4;
+constexpr long long EW_FEW = 64 * 256 * EW_U;
 
 __device__ __forceinline__ float prelu1(float v, float s) { return v >= 0.f ? v : s * v; }
 
+template <int U>
 __global__ void __launch_bounds__(256) k_prelu_fwd(const float* __restrict__ x,
                                                    const float* __restrict__ a,
                                                    float* __restrict__ y, long long n, int vec) {
@@ -221,13 +225,13 @@ __global__ void __launch_bounds__(256) k_prelu_fwd(const float* __restrict__ x,
   const long long stride = (long long)gridDim.x * blockDim.x;
   const long long t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const float4* x4 = reinterpret_cast<const float4*>(x);
-  for (long long i = blockIdx.x * (256LL * EW_U) + threadIdx.x; i < n4; i += stride * EW_U) {
-    float4 v[EW_U];
+  for (long long i = blockIdx.x * (256LL * U) + threadIdx.x; i < n4; i += stride * U) {
+    float4 v[U];
 #pragma unroll
-    for (int u = 0; u < EW_U; ++u)
+    for (int u = 0; u < U; ++u)
       if (i + 256 * u < n4) v[u] = __ldcs(x4 + i + 256 * u);
 #pragma unroll
-    for (int u = 0; u < EW_U; ++u)
+    for (int u = 0; u < U; ++u)
       if (i + 256 * u < n4)
         reinterpret_cast<float4*>(y)[i + 256 * u] =
             make_float4(prelu1(v[u].x, s), prelu1(v[u].y, s), prelu1(v[u].z, s), prelu1(v[u].w, s));
@@ -236,6 +240,7 @@ __global__ void __launch_bounds__(256) k_prelu_fwd(const float* __restrict__ x,
 }
 
 // gx = gy * (x >= 0 ? 1 : a); partial[cta] = sum over the CTA's elements of gy * x (x < 0).
+template <int U>
 __global__ void __launch_bounds__(256) k_prelu_bwd(const float* __restrict__ x,
                                                    const float* __restrict__ a,
                                                    const float* __restrict__ gy,
@@ -251,16 +256,16 @@ __global__ void __launch_bounds__(256) k_prelu_bwd(const float* __restrict__ x,
   const long long n4 = vec ? n / 4 : 0;               // float4 body (16-byte aligned pointers)
   const long long stride = (long long)gridDim.x * blockDim.x;
   const float4 *x4 = reinterpret_cast<const float4*>(x), *g4 = reinterpret_cast<const float4*>(gy);
-  for (long long i = blockIdx.x * (256LL * EW_U) + threadIdx.x; i < n4; i += stride * EW_U) {
-    float4 v[EW_U], g[EW_U];
+  for (long long i = blockIdx.x * (256LL * U) + threadIdx.x; i < n4; i += stride * U) {
+    float4 v[U], g[U];
 #pragma unroll
-    for (int u = 0; u < EW_U; ++u)
+    for (int u = 0; u < U; ++u)
       if (i + 256 * u < n4) {
         v[u] = __ldcs(x4 + i + 256 * u);
         g[u] = __ldcs(g4 + i + 256 * u);
       }
 #pragma unroll
-    for (int u = 0; u < EW_U; ++u)
+    for (int u = 0; u < U; ++u)
       if (i + 256 * u < n4) {
         float4 o;
         o.x = one(v[u].x, g[u].x);
@@ -668,7 +673,9 @@ shl_status shl_nn_prelu_forward(const float* x, const float* a, float* y, long l
   if (!x || !a || !y || n < 0) return nn_fail(SHL_EINVAL, "prelu_forward: bad arguments");
   if (n == 0) return SHL_OK;
   const int vec = aligned16(x) && aligned16(y);
-  k_prelu_fwd<<<blocks(vec ? (n + 3) / 4 : n, vec ? 256 * EW_U : 256), 256, 0, S(stream)>>>(x, a, y, n, vec);
+  if (!vec) k_prelu_fwd<1><<<blocks(n, 256), 256, 0, S(stream)>>>(x, a, y, n, 0);
+  else if (n / 4 < EW_FEW) k_prelu_fwd<1><<<blocks((n + 3) / 4, 256), 256, 0, S(stream)>>>(x, a, y, n, 1);
+  else k_prelu_fwd<EW_U><<<blocks((n + 3) / 4, 256 * EW_U), 256, 0, S(stream)>>>(x, a, y, n, 1);
   return nn_launch("prelu_forward");
 }
 
@@ -682,7 +689,8 @@ shl_status shl_nn_prelu_backward(const float* x, const float* a, const float* gy
   if (!x || !a || !gy || !gx || !ga || !ws || n < 0) return nn_fail(SHL_EINVAL, "prelu_backward: bad arguments");
   const int g = std::max(1, std::min(RED_CTAS, blocks(n, 256)));
   const int vec = aligned16(x) && aligned16(gy) && aligned16(gx);
-  k_prelu_bwd<<<g, 256, 0, S(stream)>>>(x, a, gy, gx, ws, n, vec);
+  if (!vec || n / 4 < EW_FEW) k_prelu_bwd<1><<<g, 256, 0, S(stream)>>>(x, a, gy, gx, ws, n, vec);
+  else k_prelu_bwd<EW_U><<<g, 256, 0, S(stream)>>>(x, a, gy, gx, ws, n, 1);
   k_sum<<<1, 256, 0, S(stream)>>>(ws, g, ga);
   return nn_launch("prelu_backward");
 }
