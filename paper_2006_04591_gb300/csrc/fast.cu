@@ -1176,9 +1176,9 @@ static cudaError_t r2c_t(InMode mode, bool th, bool coeffs, const RowsTArgs& a, 
     k_rows_r2c_t<LOG_M, INM, TH, PK><<<grid, P::THREADS, sm, st>>>(a);               \
   } while (0)
   constexpr bool PC = rows_packed<LOG_M>();
-  if (mode == IN_MASKED) SHL_LAUNCH(IN_MASKED, false, false);
+  if (mode == IN_MASKED) { if (th) return cudaErrorInvalidValue; SHL_LAUNCH(IN_MASKED, false, false); }
   else if (mode == IN_BF16) { if (th) SHL_LAUNCH(IN_BF16, true, PC); else SHL_LAUNCH(IN_BF16, false, PC); }
-  else if (!coeffs) SHL_LAUNCH(IN_F32, false, false);
+  else if (!coeffs && !th) SHL_LAUNCH(IN_F32, false, false);     // an image; a threshold means coefficients
   else { if (th) SHL_LAUNCH(IN_F32, true, PC); else SHL_LAUNCH(IN_F32, false, PC); }
 #undef SHL_LAUNCH
   return cudaGetLastError();
