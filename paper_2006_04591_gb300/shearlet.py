@@ -123,7 +123,8 @@ def _ptr(t):
 def current_stream_ptr(device):
     """The cudaStream_t (an int) of torch's current stream on ``device`` (a torch
     device or an index), without the Stream object that
-    torch.cuda.current_stream() builds around it on every call."""
+    torch.cuda.current_stream() builds around it on every call (with it, in a torch
+    that does not have the raw call)."""
     import torch
     if isinstance(device, int):
         index = device
@@ -133,7 +134,8 @@ def current_stream_ptr(device):
         raise ValueError("expected a CUDA device, got %s" % device)
     if index is None:
         index = torch.cuda.current_device()
-    return torch._C._cuda_getCurrentRawStream(index)
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    return raw(index) if raw is not None else torch.cuda.current_stream(index).cuda_stream
 
 
 def _stream(stream, device):
