@@ -29,3 +29,21 @@ def test_forward(n, A, D, B):
         tol = 1e-6 * n * x[b].abs().max().item() + 1e-6 * np.abs(want[b]).max()
         assert np.abs(p[b].cpu().numpy() - want[b]).max() <= tol
         assert torch.equal(op.forward(x[b:b + 1])[0], p[b])
+
+
+# Adjoint: tiles of staged bins with one and two images per CTA (600 x 600; 545 is the
+# smallest), and the untiled kernel with two pixels per thread and one, two and four
+# images (400 x 400; 9001 bins are too narrow for a staging).
+@pytest.mark.parametrize("n,A,D,B", [(600, 5, 849, 1), (600, 5, 849, 2), (600, 4, 849, 3), (545, 3, 400, 1),
+                                     (400, 4, 566, 1), (400, 4, 566, 2), (400, 3, 566, 4), (600, 3, 9001, 1)])
+def test_adjoint(n, A, D, B):
+    from paper_2006_04591_gb300.ray import RayTransform
+    op = RayTransform(n, A, D, device=0)
+    y = _randn(B, A, D)
+    g = op.adjoint(y)
+    want = R.adjoint(y.cpu().numpy(), n)
+    bins = 3 * max(1.0, D / (np.sqrt(2) * n))           # bins whose rays touch a pixel
+    for b in range(B):
+        tol = 1e-6 * n * y[b].abs().max().item() * (2.9 / n) * bins * A + 1e-6 * np.abs(want[b]).max()
+        assert np.abs(g[b].cpu().numpy() - want[b]).max() <= tol
+        assert torch.equal(op.adjoint(y[b:b + 1])[0], g[b])
