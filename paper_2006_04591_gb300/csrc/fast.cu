@@ -273,10 +273,12 @@ __device__ __forceinline__ void r2c_tile_finish(float2 (&v)[RowsT<LOG_M>::R], fl
   __syncthreads();
 }
 
-// Coefficient rows use packed additions up to M = 512 (R2C 294 -> 284 us, C2R 268 ->
-// 262 us at 16 x 512^2, K = 49); at 1024 they cost (763 -> 780 us at 8 x 1024^2).
+// Coefficient rows use packed additions from M = 128 to 512 (R2C 294 -> 284 us, C2R 268 ->
+// 262 us at 16 x 512^2, K = 49); at 1024 they cost (763 -> 780 us at 8 x 1024^2), and below
+// 128 as well (64 x 256 x 64, K = 17: decomposition 77.9 -> 79.6 us, reconstruction
+// 102.7 -> 105.1 us).
 template <int LOG_M>
-__host__ __device__ constexpr bool rows_packed() { return LOG_M < 10; }
+__host__ __device__ constexpr bool rows_packed() { return LOG_M >= 7 && LOG_M < 10; }
 
 // PK: packed additions (coefficient rows; the image's rows feed the bfloat16
 // decomposition as well and keep the scalar form).
