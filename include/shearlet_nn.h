@@ -45,8 +45,9 @@ shl_status shl_nn_conv3x3_backward_weight(const float* in, const float* gout, fl
  * (inputs and weights rounded to nearest even), float32 accumulation, so
  * the result equals the convolution of the bfloat16-rounded tensors up to
  * float32 summation order.  Supported when shl_nn_conv3x3_tc_supported()
- * (1 <= Ci, Co <= 48 and W a multiple of 128) and the input (gout for the
- * backward call) is 16-byte aligned; SHL_EINVAL otherwise. */
+ * (Ci, Co <= 48, or 112 inputs and 32 outputs, or 32 and 112; W even, at least
+ * 16) and the input (gout for the backward call) is 16-byte aligned; SHL_EINVAL
+ * otherwise. */
 int shl_nn_conv3x3_tc_supported(int Ci, int Co, int H, int W);
 shl_status shl_nn_conv3x3_forward_tc(const float* in, const float* w, const float* bias,
                                      float* out, int B, int Ci, int Co, int H, int W,
@@ -59,8 +60,8 @@ shl_status shl_nn_conv3x3_backward_data_tc(const float* gout, const float* w, fl
  * gout x shifted input with both rounded to bfloat16, float32 accumulation
  * (per-CTA partials in ws, summed in a fixed order); gb (may be NULL) in
  * float32 from the unrounded gout.  Supported when
- * shl_nn_conv3x3_wgrad_tc_supported() (3 Ci <= 128, Co <= 48, W a multiple
- * of 128) and in, gout are 16-byte aligned; ws holds
+ * shl_nn_conv3x3_wgrad_tc_supported() (3 Ci <= 128, Co <= 96, W even, at
+ * least 16) and in, gout are 16-byte aligned; ws holds
  * shl_nn_conv3x3_backward_weight_tc_workspace_floats() floats. */
 int shl_nn_conv3x3_wgrad_tc_supported(int Ci, int Co, int H, int W);
 size_t shl_nn_conv3x3_backward_weight_tc_workspace_floats(int B, int Ci, int Co, int H, int W);

@@ -13,8 +13,9 @@
 // (K = 49, float32, decomposition and reconstruction): 16 x 480 x 640 5375 -> 1806 us
 // (column pass of the reconstruction 1864 -> 395, of the decomposition 1124 -> 417,
 // row passes 1166 -> 452 and 1127 -> 517), 16 x 500^2 4345 -> 1503 us, 4 x 509^2
-// (Bluestein, P = 1024) 3992 -> 1262 us; with K = 17, 16 x 222 x 301 (Bluestein,
-// P = 512 and 1024) 1575 -> 599 us.
+// (Bluestein, P = 1024) 3992 -> 1262 us; with packed additions and the group sums below
+// 1620, 1420 and 1152 us.  With K = 17, 16 x 222 x 301 (Bluestein, P = 512 and 1024)
+// 1575 -> 599 us.
 // At 480 x 640 the passes now run at 35-55 % of the DRAM rate of the planes and
 // coefficients that they move; what is left is latency at 18 to 24 warps per SM.
 //

@@ -5,7 +5,7 @@
 //                  to four images: Joseph's method, one linear-interpolation
 //                  sample per pixel row (or column), the rows it samples
 //                  staged in shared memory with the images interleaved.
-//   k_ray_adjoint  two pixels and up to four images per thread: for each angle,
+//   k_ray_adjoint  one or two pixels and up to four images per thread: for each angle,
 //                  the bins whose rays sample this pixel's row (column) near
 //                  it, with the forward's own weights.
 //
@@ -70,8 +70,9 @@ template <> struct __align__(8) Vec<2> { float v[2]; };
 template <> struct __align__(16) Vec<4> { float v[4]; };
 
 // ---------------------------------------------------------------- forward
-// What bounds it: shared-memory reads, two NB-wide words per sample.  Reading
-// the image through L1 instead, one ray per thread, cost a gather of up to 32
+// What bounds it: the wait for the staged pixels and two barriers per staging, at two to
+// four CTAs per SM (8 images of 512 x 512, 60 angles: issue 57 %, shared memory 39 % of
+// its rate).  Reading the image through L1 instead, one ray per thread, cost a gather of up to 32
 // lines per load at the angles sampled by columns; staging T rows (or, transposed,
 // T columns) of the pixels that the CTA's rays cross makes both kinds of angle
 // the same, interleaving NB images shares the position and the weights between
@@ -307,8 +308,8 @@ __global__ void __launch_bounds__(256) k_ray_adjoint(const float* __restrict__ s
 
 // The same with the bins that a tile of 32 x 32 pixels can receive staged in shared
 // memory, images interleaved: one NB-wide read per bin in place of NB gathers
-// through L1 (measured as above 527 -> 277 us, 296 us with the exact weights).  Chunks
-// of `ac` angles, W bins each, from bin s_lo on.
+// through L1 (measured as above 527 -> 277 us, 296 us with the exact weights; bound by
+// issue, 79 %).  Chunks of `ac` angles, W bins each, from bin s_lo on.
 constexpr int ADJ_TILE_PIX = 4;    // pixels per thread, 8 rows apart
 constexpr int ADJ_CHUNK = 16;      // most angles staged at a time
 constexpr size_t ADJ_SMEM = 48 * 1024;
