@@ -72,10 +72,10 @@ template <> struct __align__(16) Vec<4> { float v[4]; };
 // ---------------------------------------------------------------- forward
 // What bounds it: the wait for the staged pixels and two barriers per staging, at two to
 // four CTAs per SM (8 images of 512 x 512, 60 angles: issue 57 %, shared memory 39 % of
-// its rate).  Reading the image through L1 instead, one ray per thread, cost a gather of up to 32
-// lines per load at the angles sampled by columns; staging T rows (or, transposed,
-// T columns) of the pixels that the CTA's rays cross makes both kinds of angle
-// the same, interleaving NB images shares the position and the weights between
+// its rate).  Reading the image through L1 instead, one ray per thread, cost a gather
+// of up to 32 lines per load at the angles sampled by columns; staging T rows (or,
+// transposed, T columns) of the pixels that the CTA's rays cross makes both kinds of
+// angle the same, interleaving NB images shares the position and the weights between
 // them, and two neighbouring angles share one staging.  Measured at 8 images of
 // 512 x 512, 180 angles, 725 bins: 1402 us with one thread per ray, 338 us so (one
 // image: 239 and 121 us).
@@ -222,13 +222,12 @@ __global__ void __launch_bounds__(FWD_BINS) k_ray_forward(const float* __restric
 // ---------------------------------------------------------------- adjoint
 // Pixel (t, k) of angle a receives every bin d with |u(d, t) - k| < 1, with the
 // forward's own weight, rounding included (hat_weight), so that the two are exact
-// transposes.  The bins start at
-// the one below the fractional bin of u = k - 1; ADJ_MARGIN covers the rounding
-// of that bin (below 0.01 over the accepted sizes).  What bounds it: the
-// bins' reads through L1, shared by nothing but the four images' position, weights
-// and address.  Measured as above: 1770 us with one thread
-// per pixel and image (a floor and a compare per candidate bin), 527 us so; 32
-// images of 128 x 128 at 30 angles: 96 and 33 us (forward 107 and 45 us).
+// transposes.  The bins start at the one below the fractional bin of u = k - 1;
+// ADJ_MARGIN covers the rounding of that bin (below 0.01 over the accepted sizes).
+// What bounds it: the bins' reads through L1, shared by nothing but the four images'
+// position, weights and address.  Measured as above: 1770 us with one thread per pixel
+// and image (a floor and a compare per candidate bin), 527 us so; 32 images of 128 x 128
+// at 30 angles: 95 and 35 us (forward 107 and 41 us).
 constexpr float ADJ_MARGIN = 0.05f;
 constexpr int ADJ_PIX = 2;         // pixels per thread, 8 rows apart; one where that leaves
                                    // SMs without two CTAs (16^2, 8 angles, 2000
